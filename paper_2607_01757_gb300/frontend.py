@@ -119,10 +119,10 @@ class FrontEnd:
 
     def launches_per_step(self):
         """Kernel launches of one step after the first (batched runs as
-        reported by vt_batch_info; 7 per detector call)."""
+        reported by vt_batch_info; 3 per detector call)."""
         a = vt.vt_batch_info(self.batch_a)["launches_per_run"]
         b = vt.vt_batch_info(self.batch_b)["launches_per_run"] if any(sp.stereo for sp in self.specs) else 0
-        return a + 1 + 7 * ((len(self.specs) + 63) // 64) + b + 1
+        return a + 1 + 3 * ((len(self.specs) + 63) // 64) + b + 1
 
     def pool(self, k):
         """(positions, identities, ages) of stream k's pool, on the host."""
