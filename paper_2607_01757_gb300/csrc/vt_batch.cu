@@ -28,8 +28,8 @@ template <int WIN, int GT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, KltOcc<WIN>::min_blocks * 4 / WARPS)
     k_klt_batch(const uint8_t *tab, int *counter) {
     extern __shared__ __align__(16) uint8_t klt_smem[];
-    KSmem<WIN> &sm = reinterpret_cast<KSmem<WIN> *>(klt_smem)[threadIdx.x >> 5];
-    ksmem_init<WIN>(sm, threadIdx.x & 31);
+    KCta<WIN> &C = kcta_init<WIN>(klt_smem);
+    KSmem<WIN> &sm = C.warp[threadIdx.x >> 5];
     const BatchHdr *H = reinterpret_cast<const BatchHdr *>(tab);
     const BTask *tasks = reinterpret_cast<const BTask *>(tab + H->off_tasks);
     const int *p0s = reinterpret_cast<const int *>(tab + H->off_prefix);
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(WARPS * 32, KltOcc<WIN>::min_blocks * 4 / WARP
         KParams Pt = P;
         Pt.levels = t.levels;
         KOut o;
-        track_point_dir<WIN, GT, false>(t.I, t.J, Pt, u.x, u.y, t.fb != 0, false, 0.f, 0.f, lane, sm, o);
+        track_point_dir<WIN, GT, false>(t.I, t.J, Pt, u.x, u.y, t.fb != 0, false, 0.f, 0.f, lane, C, sm, o);
         if (lane == 0) {
             if (o.reason == kReasonPending) {  // left to k_klt_batch_f64
                 t.status[i] = kStatusPending;
@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(WARPS * 32, KltOcc<WIN>::min_blocks * 4 / WARP
 template <int WIN, int GT>
 __global__ void __launch_bounds__(128) k_klt_batch_f64(const uint8_t *tab) {
     extern __shared__ __align__(16) uint8_t klt_smem[];
-    KSmem<WIN> &sm = reinterpret_cast<KSmem<WIN> *>(klt_smem)[threadIdx.x >> 5];
-    ksmem_init<WIN>(sm, threadIdx.x & 31);
+    KCta<WIN> &C = kcta_init<WIN>(klt_smem);
+    KSmem<WIN> &sm = C.warp[threadIdx.x >> 5];
     const BatchHdr *H = reinterpret_cast<const BatchHdr *>(tab);
     const BTask *tasks = reinterpret_cast<const BTask *>(tab + H->off_tasks);
     const int *p0s = reinterpret_cast<const int *>(tab + H->off_prefix);
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(128) k_klt_batch_f64(const uint8_t *tab) {
         KParams Pt = P;
         Pt.levels = t.levels;
         KOut o;
-        track_point_dir<WIN, GT, true>(t.I, t.J, Pt, u.x, u.y, t.fb != 0, false, 0.f, 0.f, lane, sm, o);
+        track_point_dir<WIN, GT, true>(t.I, t.J, Pt, u.x, u.y, t.fb != 0, false, 0.f, 0.f, lane, C, sm, o);
         if (lane == 0) {
             t.pts_out[i] = make_float2(o.x, o.y);
             t.status[i] = (uint8_t)o.status;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(128) k_klt_batch_f64(const uint8_t *tab) {
 
 template <int WIN, int GT>
 static void launch_f64_win(const uint8_t *tab, int grid, cudaStream_t s) {
-    const size_t smem = 4 * sizeof(KSmem<WIN>);
+    const size_t smem = KCta<WIN>::bytes(4);
     static const bool attr = [smem] {  // once, thread-safe static initialisation
         return cudaFuncSetAttribute(k_klt_batch_f64<WIN, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem) == cudaSuccess;
@@ -154,7 +154,7 @@ struct KltBatchKernel {
 
 template <int WIN, int GT, int WARPS>
 static KltBatchKernel klt_batch_entry() {
-    const size_t smem = WARPS * sizeof(KSmem<WIN>);
+    const size_t smem = KCta<WIN>::bytes(WARPS);
     // opt in to more than 48 KB where needed (once, thread-safe static initialisation)
     static const bool attr = [smem] {
         return cudaFuncSetAttribute(k_klt_batch<WIN, GT, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,

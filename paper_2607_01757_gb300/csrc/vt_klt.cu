@@ -29,8 +29,8 @@ struct KltArgs {
 template <int WIN, int GT, bool FB, bool F64>
 __global__ void __launch_bounds__(KLT_WARPS * 32, KltOcc<WIN>::min_blocks) k_klt(const __grid_constant__ KltArgs A) {
     extern __shared__ __align__(16) uint8_t klt_smem[];
-    KSmem<WIN> &sm = reinterpret_cast<KSmem<WIN> *>(klt_smem)[threadIdx.x >> 5];
-    ksmem_init<WIN>(sm, threadIdx.x & 31);
+    KCta<WIN> &C = kcta_init<WIN>(klt_smem);
+    KSmem<WIN> &sm = C.warp[threadIdx.x >> 5];
     const int pt = blockIdx.x * KLT_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (pt >= A.n) return;
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(KLT_WARPS * 32, KltOcc<WIN>::min_blocks) k_klt
     float2 g = make_float2(0.f, 0.f);
     const bool hg = !FB && A.guess != nullptr;
     if (hg) g = A.guess[pt];
-    track_point_dir<WIN, GT, F64>(A.I.lv, A.J.lv, A.P, p.x, p.y, FB, hg, g.x, g.y, lane, sm, o);
+    track_point_dir<WIN, GT, F64>(A.I.lv, A.J.lv, A.P, p.x, p.y, FB, hg, g.x, g.y, lane, C, sm, o);
     if (!F64 && o.reason == kReasonPending) {
         if (lane == 0) A.status[pt] = kStatusPending;
         return;
@@ -69,7 +69,7 @@ __global__ void k_fb_check(const float2 *p0, const float2 *p1, const uint8_t *sf
 template <int WIN, int GT, bool FB, bool F64>
 static void launch_pass(const KltArgs &A, cudaStream_t s) {
     const int blocks = (A.n + KLT_WARPS - 1) / KLT_WARPS;
-    const size_t smem = KLT_WARPS * sizeof(KSmem<WIN>);
+    const size_t smem = KCta<WIN>::bytes(KLT_WARPS);
     if (smem > 48 * 1024) {
         static const bool attr = [smem] {  // once, thread-safe static initialisation
             return cudaFuncSetAttribute(k_klt<WIN, GT, FB, F64>, cudaFuncAttributeMaxDynamicSharedMemorySize,

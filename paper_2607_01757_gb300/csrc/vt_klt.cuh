@@ -22,7 +22,8 @@
 // iterations that stay in the same cell reuse the moments.  The template and
 // its gradients stay in registers (three floats per owned sample); the image and
 // gradient window it is sampled from, and each footprint, are staged in
-// per-warp shared memory by cp.async.  Sums over the window are per-lane FP32
+// per-warp shared memory by cp.async, a level's template while the level
+// before it iterates and its first footprint while its template is sampled.  Sums over the window are per-lane FP32
 // sums over rows followed by a warp reduction that leaves bit-identical
 // totals in every lane (an XOR butterfly, or a reduce-scatter and broadcast),
 // so control flow stays warp-uniform.
@@ -153,38 +154,46 @@ __device__ __forceinline__ float kdiff(float a, float b, float c, float d) {
 // 2^-l exactly.
 __device__ __forceinline__ float pow2neg(int l) { return __int_as_float((127 - l) << 23); }
 
-// Per-warp shared scratch: the staged (win + 1)^2 window of a level image --
-// the footprint of J for one sweep, or the template's source -- in win + 1
-// rows of NC 16-byte chunks, and the template's gradient window in win + 1
-// rows of NG 16-byte chunks.
+// Per-warp shared scratch: the staged (win + 1)^2 windows -- the footprint of J
+// for one sweep, and the template's image and gradient windows of this level
+// and of the next one (levels alternate between the two buffers, so the next
+// level's template is copied in while this level iterates) -- in win + 1 rows
+// of NC (image) or NG (gradients) 16-byte chunks.
 template <int WIN>
 struct KSmem {
     static constexpr int NC = (WIN + 31) / 16;  // 16-byte chunks per staged row: cover 15 + win + 1 bytes
     static constexpr int JS = NC * 16;          // staged row stride in bytes
-    static_assert(JS >= 15 + WIN + 1 && JS - 1 - WIN <= 32, "a staged row covers the footprint row and reads "
-                                                              "at most 32 bytes past it (the allocation keeps 256)");
-    uint8_t j[(WIN + 1) * JS];
+    static_assert(JS >= 15 + WIN + 1, "a staged row covers the footprint row");
     static constexpr int NG = (4 * (3 + WIN + 1) + 15) / 16;  // 16-byte chunks per staged gradient row
     static constexpr int GS = NG * 4;                         // staged gradient row stride in words
-    static_assert(GS >= 3 + WIN + 1 && 4 * (GS - WIN - 1) <= 32, "a staged gradient row covers the window row "
-                                                                 "and reads at most 32 bytes past it");
-    uint32_t g[(WIN + 1) * GS];
-    uint8_t t[(WIN + 1) * JS];  // the template's image window, kept while footprints are staged (FP64 levels)
-    // zeros that a lane's run outside the window reads instead of the staged
-    // windows (its template samples and error terms are then exactly zero
-    // without a select per sample): RL + 1 rows of two bytes / words at the
-    // staged strides (RL = samples per run)
-    static constexpr int RLZ = WIN / (WIN == 31 ? 1 : 3);
-    uint8_t zj[RLZ * JS + 16];
-    uint32_t zg[RLZ * GS + 4];
+    static_assert(GS >= 3 + WIN + 1, "a staged gradient row covers the window row");
+    uint8_t j[(WIN + 1) * JS];
+    uint8_t t[2][(WIN + 1) * JS];
+    uint32_t g[2][(WIN + 1) * GS];
 };
 
-// Clear a warp's zero rows (once per kernel, before the first point).
+// Shared scratch of a CTA: its warps' windows, and zeros that a lane's run
+// outside the window reads instead of the staged windows (its template
+// samples and error terms are then exactly zero without a select per sample):
+// a run's rows of two bytes / words at the staged strides.
 template <int WIN>
-__device__ __forceinline__ void ksmem_init(KSmem<WIN> &sm, int lane) {
-    for (int k = lane; k < (int)sizeof(sm.zj); k += 32) sm.zj[k] = 0;
-    for (int k = lane; k < (int)(sizeof(sm.zg) / 4); k += 32) sm.zg[k] = 0;
-    __syncwarp();
+struct KCta {
+    static constexpr int RLZ = WIN / (WIN == 31 ? 1 : 3);
+    uint8_t zj[RLZ * KSmem<WIN>::JS + 16];
+    uint32_t zg[RLZ * KSmem<WIN>::GS + 4];
+    KSmem<WIN> warp[1];  // one per warp of the CTA
+
+    static constexpr size_t bytes(int warps) { return sizeof(KCta) + (warps - 1) * sizeof(KSmem<WIN>); }
+};
+
+// Clear the zero rows (every thread of the CTA, once per kernel).
+template <int WIN>
+__device__ __forceinline__ KCta<WIN> &kcta_init(uint8_t *smem) {
+    KCta<WIN> &C = *reinterpret_cast<KCta<WIN> *>(smem);
+    for (int k = threadIdx.x; k < (int)sizeof(C.zj); k += blockDim.x) C.zj[k] = 0;
+    for (int k = threadIdx.x; k < (int)(sizeof(C.zg) / 4); k += blockDim.x) C.zg[k] = 0;
+    __syncthreads();
+    return C;
 }
 
 // Which window samples a lane owns.  The win x win window is cut into runs
@@ -225,8 +234,8 @@ __device__ __forceinline__ void run_of(int lane, int i, int &c, int &r0, bool &v
 // (c <= win) computes the raw Scharr responses of staged column c -- the
 // integers the pyramid kernels would have stored for the replicate-clamped
 // pixel (reflect-101 neighbours) -- and stores them as int16 pairs in the
-// staged gradient window, with the pixel itself in the staged image window,
-// so the template is then sampled exactly as from stored int16 gradients.
+// staged gradient window, with the pixel itself in the staged image window
+// (column c of the window at staged column c), so the template is then sampled exactly as from stored int16 gradients.
 //
 // Per image row y the lane forms d(y) = I(y, x+1) - I(y, x-1) and
 // s(y) = 3 I(y, x-1) + 10 I(y, x) + 3 I(y, x+1); the gradient of row y is
@@ -236,7 +245,7 @@ __device__ __forceinline__ void run_of(int lane, int i, int &c, int &r0, bool &v
 // image's first or last line takes its reflected neighbour (row 1 or h-2)
 // on both sides instead.
 template <int WIN>
-__device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0, int lane, KSmem<WIN> &sm) {
+__device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0, int lane, uint8_t *st, uint32_t *sg) {
     constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS;
     const bool ld = lane <= WIN;
     const int q = clampi(x0 + lane, 0, L.w - 1);
@@ -256,8 +265,8 @@ __device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0,
     };
     // reflected neighbours of the first and last image rows (used only when
     // the window reaches them)
-    int dt = 0, st = 0, db = 0, sb = 0, unused;
-    if (y0 <= 0 || hm1 == 0) terms(refl101(-1, L.h), dt, st, unused);
+    int dt = 0, s_t = 0, db = 0, sb = 0, unused;
+    if (y0 <= 0 || hm1 == 0) terms(refl101(-1, L.h), dt, s_t, unused);
     if (y0 + WIN >= hm1) terms(refl101(L.h, L.h), db, sb, unused);
     int dm, sm_m, cm, d0, s0, c0;
     terms(clampi(y0 - 1, 0, hm1), dm, sm_m, cm);
@@ -269,12 +278,12 @@ __device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0,
         int dp, sp, cp;
         terms(clampi(y0 + r + 1, 0, hm1), dp, sp, cp);
         const bool top = yc == 0, bot = yc == hm1;
-        const int du = top ? dt : (bot ? db : dm), su = top ? st : (bot ? sb : sm_m);
-        const int dd = top ? dt : (bot ? db : dp), sd = top ? st : (bot ? sb : sp);
+        const int du = top ? dt : (bot ? db : dm), su = top ? s_t : (bot ? sb : sm_m);
+        const int dd = top ? dt : (bot ? db : dp), sd = top ? s_t : (bot ? sb : sp);
         const int gx = 3 * (du + dd) + 10 * d0, gy = sd - su;
         if (ld) {
-            sm.j[r * JS + lane] = (uint8_t)c0;
-            sm.g[r * GS + lane] = (uint32_t)(uint16_t)(int16_t)gx | ((uint32_t)(uint16_t)(int16_t)gy << 16);
+            st[r * JS + lane] = (uint8_t)c0;
+            sg[r * GS + lane] = (uint32_t)(uint16_t)(int16_t)gx | ((uint32_t)(uint16_t)(int16_t)gy << 16);
         }
         dm = d0;
         sm_m = s0;
@@ -285,81 +294,119 @@ __device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0,
     __syncwarp();
 }
 
-// Sample the template of level `L` around (ux, uy) at the lane's window
-// samples (KRuns): T and its gradients, zero for samples outside the
-// window.  The (win + 1)^2 image and gradient footprint is first staged in
-// shared memory (16-byte cp.async chunks of each clamped row when the
-// columns lie inside the level -- they may read up to 26 image bytes (window
-// 21; at most 30 for any window) and 24 gradient bytes past a row's last
-// pixel, inside the pitch, the pyramid allocation's slack, or the 32 bytes a
-// caller-owned level 0 keeps readable after its last row -- else one clamped
-// column per lane; computed in place for a level without gradient planes).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// All but the newest N groups of this thread have arrived.
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// Start copying win + 1 rows of NCH 16-byte chunks (row pitch `pitch` bytes,
+// rows y0 .. y0 + win clamped to 0 .. hm1) from `base` to `dst`, the chunks
+// below `chunks` of each row.  32 / NCH rows go per step, a lane keeping one
+// chunk of a row: its addresses advance by a constant per step, two
+// instructions per copied chunk (an index split into row and chunk per copy
+// took about 18).
+template <int WIN, int NCH>
+__device__ __forceinline__ void copy_rows(uint32_t dst, const uint8_t *base, int pitch, int y0, int hm1, int chunks,
+                                          int lane) {
+    constexpr int RS = 32 / NCH, STEPS = (WIN + RS) / RS;  // rows per step; steps for win + 1 rows
+    const int r = lane / NCH, c = lane - r * NCH;
+    const uint32_t d = dst + 16 * lane;
+    const int rows = r < RS && c < chunks ? WIN + 1 - r : 0;  // the lane copies rows r + k RS, k RS < rows
+    if (y0 >= 0 && y0 + WIN <= hm1) {
+        const uint8_t *src = base + (size_t)(y0 + r) * pitch + 16 * c;
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            if (k * RS < rows) cp_async16(d + k * RS * NCH * 16, src);
+            src += RS * pitch;
+        }
+    } else {
+#pragma unroll 1
+        for (int k = 0; k < STEPS; ++k)
+            if (k * RS < rows)
+                cp_async16(d + k * RS * NCH * 16, base + (size_t)clampi(y0 + r + k * RS, 0, hm1) * pitch + 16 * c);
+    }
+}
+
+// First staged column of a window whose leftmost column is x0: the aligned
+// column (16 image bytes, 4 gradient words) at or before the first one inside
+// the level.
+__device__ __forceinline__ int staged_x(int x0, int align) { return max(x0, 0) & ~(align - 1); }
+
+// Start staging the (win + 1)^2 image window with top-left (x0, y0) at `st`
+// (and, with GRAD, the gradient window at `sg`): each row, clamped into the
+// level, in whole aligned 16-byte chunks from staged_x on, by cp.async (no
+// register round trip; the caller commits and waits).  Chunks that begin
+// past the level's last column are left out; the last one may read up to 15
+// bytes past it, inside the row's pitch.  Columns outside the level are not
+// staged: the readers clamp theirs (run_columns).
+template <int WIN, bool GRAD>
+__device__ __forceinline__ void stage_window(const Level &L, int x0, int y0, int lane, uint8_t *st, uint32_t *sg) {
+    const int hm1 = L.h - 1, wx = staged_x(x0, 16);
+    __syncwarp();  // every lane is done with what the buffers held
+    copy_rows<WIN, KSmem<WIN>::NC>((uint32_t)__cvta_generic_to_shared(st), L.img + wx, L.pitch, y0, hm1,
+                                   (L.w - wx + 15) >> 4, lane);
+    if constexpr (GRAD) {
+        const int gw = staged_x(x0, 4);
+        copy_rows<WIN, KSmem<WIN>::NG>((uint32_t)__cvta_generic_to_shared(sg),
+                                       reinterpret_cast<const uint8_t *>(L.grad + gw), L.gpitch * 4, y0, hm1,
+                                       (L.w - gw + 3) >> 2, lane);
+    }
+}
+
+// Stage the footprint of J with top-left (x0, y0) and wait for it (and for
+// every copy under way).
+template <int WIN>
+__device__ __forceinline__ void stage_footprint(const Level &L, int x0, int y0, int lane, KSmem<WIN> &sm) {
+    stage_window<WIN, false>(L, x0, y0, lane, sm.j, nullptr);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+}
+
+// Where a run's column c and its right neighbour lie in a staged row
+// (replicate-clamped into 0 .. w - 1): offsets from the first staged column.
+template <int WIN>
+__device__ __forceinline__ void run_columns(int x0, int w, int sx, int c, int &o0, int &o1) {
+    o0 = x0 + c - sx;
+    o1 = o0 + 1;
+    if (x0 < 0 || x0 + WIN >= w) {
+        o0 = clampi(x0 + c, 0, w - 1) - sx;
+        o1 = clampi(x0 + c + 1, 0, w - 1) - sx;
+    }
+}
+
+// The template at the lane's window samples (KRuns): T and its gradients,
+// sampled at fractional offset (ax, ay) from the staged windows, zero for
+// samples outside the window.
 template <int WIN, int GT>
-__device__ __forceinline__ void load_template(const Level &L, float ux, float uy, int lane,
-                                              float (&T)[KRuns<WIN>::NS], float (&GX)[KRuns<WIN>::NS],
-                                              float (&GY)[KRuns<WIN>::NS], KSmem<WIN> &sm, int &offi, int &offg) {
-    constexpr int HW = WIN / 2;
-    constexpr int NC = KSmem<WIN>::NC, JS = KSmem<WIN>::JS, NG = KSmem<WIN>::NG, GS = KSmem<WIN>::GS;
-    constexpr int RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
+__device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_t *st, const uint32_t *sg, int x0,
+                                                int w, float ax, float ay, int lane, float (&T)[KRuns<WIN>::NS],
+                                                float (&GX)[KRuns<WIN>::NS], float (&GY)[KRuns<WIN>::NS]) {
+    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     // staged gradient words are int16 pairs when computed in place
     constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
-    const float fx = floorf(ux), fy = floorf(uy);
-    const float ax = ux - fx, ay = uy - fy;
-    const int x0 = (int)fx - HW, y0 = (int)fy - HW;
-    const int hm1 = L.h - 1;
-    __syncwarp();
-    if constexpr (GT == VT_GRAD_NONE) {
-        offi = offg = 0;
-        stage_window_otf<WIN>(L, x0, y0, lane, sm);
-    } else {
-        if (x0 >= 0 && x0 + WIN < L.w) {
-            const int wx = x0 & ~15, gw = x0 & ~3;
-            offi = x0 - wx;
-            offg = x0 - gw;
-            const uint32_t sbj = (uint32_t)__cvta_generic_to_shared(sm.j);
-            const uint32_t sbg = (uint32_t)__cvta_generic_to_shared(sm.g);
-            for (int k = lane; k < (WIN + 1) * NC; k += 32) {
-                const int row = k / NC, c = k - row * NC;
-                const uint8_t *src = L.img + (size_t)clampi(y0 + row, 0, hm1) * L.pitch + wx + 16 * c;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sbj + row * JS + 16 * c), "l"(src)
-                             : "memory");
-            }
-            for (int k = lane; k < (WIN + 1) * NG; k += 32) {
-                const int row = k / NG, c = k - row * NG;
-                const uint32_t *src = L.grad + (size_t)clampi(y0 + row, 0, hm1) * L.gpitch + gw + 4 * c;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sbg + 4 * (row * GS + 4 * c)),
-                             "l"(src)
-                             : "memory");
-            }
-            asm volatile("cp.async.wait_all;\n" ::: "memory");
-        } else {
-            offi = offg = 0;
-            if (lane <= WIN) {
-                const int c = clampi(x0 + lane, 0, L.w - 1);
-#pragma unroll
-                for (int r = 0; r <= WIN; ++r) {
-                    const int row = clampi(y0 + r, 0, hm1);
-                    sm.j[r * JS + lane] = __ldg(L.img + (size_t)row * L.pitch + c);
-                    sm.g[r * GS + lane] = __ldg(L.grad + (size_t)row * L.gpitch + c);
-                }
-            }
-        }
-        __syncwarp();
-    }
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
         int c, r0;
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
-        const uint8_t *jr = valid ? &sm.j[r0 * JS + offi + c] : sm.zj;
-        const uint32_t *gr = valid ? &sm.g[r0 * GS + offg + c] : sm.zg;
+        int o0, o1;
+        run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
+        const uint8_t *j0 = valid ? st + r0 * JS + o0 : C.zj, *j1 = valid ? st + r0 * JS + o1 : C.zj;
+        const int dg = staged_x(x0, 16) - staged_x(x0, 4);
+        const uint32_t *g0 = valid ? sg + r0 * GS + o0 + dg : C.zg, *g1 = valid ? sg + r0 * GS + o1 + dg : C.zg;
         float pi = 0.f, pgx = 0.f, pgy = 0.f;
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(jr[r * JS]), mvr = u8f(jr[r * JS + 1]);
+            const float mv = u8f(j0[r * JS]), mvr = u8f(j1[r * JS]);
             float gx, gy, gxr, gyr;
-            unpack_grad<GTS>(gr[r * GS], gx, gy);
-            unpack_grad<GTS>(gr[r * GS + 1], gxr, gyr);
+            unpack_grad<GTS>(g0[r * GS], gx, gy);
+            unpack_grad<GTS>(g1[r * GS], gxr, gyr);
             const float hi = fmaf(ax, mvr - mv, mv);
             const float hgx = fmaf(ax, gxr - gx, gx);
             const float hgy = fmaf(ax, gyr - gy, gy);
@@ -375,45 +422,6 @@ __device__ __forceinline__ void load_template(const Level &L, float ux, float uy
     }
 }
 
-// Stage the (win + 1) x (win + 1) footprint of J with top-left (x0, y0) in
-// shared memory, rows and columns clamped into the image (replicate).  When
-// its columns lie inside the image, each (clamped) row is copied in whole
-// aligned 16-byte chunks by cp.async (global to shared, no register round
-// trip); they may read up to 26 bytes (window 21) past a row's last pixel,
-// inside the level's pitch, the pyramid allocation's slack or a caller-owned
-// level 0's 32 readable bytes after its last row.  Otherwise lane
-// c loads column c (clamped) of every row.  Returns the byte offset of column
-// 0 within a staged row.
-template <int WIN>
-__device__ __forceinline__ int stage_footprint(const Level &L, int x0, int y0, int lane, KSmem<WIN> &sm) {
-    constexpr int NC = KSmem<WIN>::NC, JS = KSmem<WIN>::JS;
-    int off;
-    __syncwarp();  // every lane is done with the previous footprint
-    if (x0 >= 0 && x0 + WIN < L.w) {
-        const int wx0 = x0 & ~15;
-        off = x0 - wx0;
-        const uint8_t *base = L.img + wx0;
-        const int hm1 = L.h - 1;
-        const uint32_t sb = (uint32_t)__cvta_generic_to_shared(sm.j);
-        for (int k = lane; k < (WIN + 1) * NC; k += 32) {
-            const int row = k / NC, wc = k - row * NC;
-            const uint8_t *g = base + (size_t)clampi(y0 + row, 0, hm1) * L.pitch + 16 * wc;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sb + row * JS + 16 * wc), "l"(g) : "memory");
-        }
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
-    } else {
-        off = 0;
-        if (lane <= WIN) {
-            const uint8_t *col = L.img + clampi(x0 + lane, 0, L.w - 1);
-            const int hm1 = L.h - 1;
-#pragma unroll
-            for (int r = 0; r <= WIN; ++r) sm.j[r * JS + lane] = __ldg(col + (size_t)clampi(y0 + r, 0, hm1) * L.pitch);
-        }
-    }
-    __syncwarp();
-    return off;
-}
-
 // Moments of one integer footprint F (top-left (x0, y0)) against the template.
 // With F00 = F(y, x), F01 = F(y, x+1), F10 = F(y+1, x), F11 = F(y+1, x+1) for
 // window sample (y, x), the bilinear sample at fractional offset (bx, by) is
@@ -423,13 +431,13 @@ __device__ __forceinline__ int stage_footprint(const Level &L, int x0, int y0, i
 //   R = sum (T - F00) grad T, Sx = sum (F01 - F00) grad T,
 //   Sy = sum (F10 - F00) grad T, Sxy = sum (F11 - F10 - F01 + F00) grad T.
 // The footprint differences are exact (integers); m[0..3] are the x parts
-// (R, Sx, Sy, Sxy against Tx), m[4..7] the y parts.
+// (R, Sx, Sy, Sxy against Tx), m[4..7] the y parts.  The footprint is staged
+// in sm.j; w: the level's width.
 template <int WIN>
-__device__ __forceinline__ void cell_moments(const Level &L, int x0, int y0, int lane,
-                                             const float (&T)[KRuns<WIN>::NS], const float (&GX)[KRuns<WIN>::NS],
-                                             const float (&GY)[KRuns<WIN>::NS], KSmem<WIN> &sm, float (&m)[8]) {
+__device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&T)[KRuns<WIN>::NS],
+                                             const float (&GX)[KRuns<WIN>::NS], const float (&GY)[KRuns<WIN>::NS],
+                                             const KSmem<WIN> &sm, float (&m)[8]) {
     constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
-    const int off = stage_footprint<WIN>(L, x0, y0, lane, sm);
     float a[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) a[k] = 0.f;
@@ -438,12 +446,14 @@ __device__ __forceinline__ void cell_moments(const Level &L, int x0, int y0, int
         int c, r0;
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);  // samples of a run outside the window weigh zero
-        const uint8_t *jr = &sm.j[r0 * JS + off + c];
+        int o0, o1;
+        run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
+        const uint8_t *j0 = &sm.j[r0 * JS + o0], *j1 = &sm.j[r0 * JS + o1];
         float pmv = 0.f, pdx = 0.f;
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(jr[r * JS]);
-            const float dx = u8f(jr[r * JS + 1]) - mv;  // F(r, c+1) - F(r, c), exact
+            const float mv = u8f(j0[r * JS]);
+            const float dx = u8f(j1[r * JS]) - mv;  // F(r, c+1) - F(r, c), exact
             if (r > 0) {
                 const int s = i * RL + r - 1;
                 const float e0 = T[s] - pmv;
@@ -466,26 +476,26 @@ __device__ __forceinline__ void cell_moments(const Level &L, int x0, int y0, int
     warp_sum8(a, lane, m);
 }
 
-// Error sweep at (qx, qy): sum |T - J_l(q + x)| over the window.
+// Error sweep over the staged footprint at fractional offset (bx, by): sum
+// |T - J(q + x)| over the window.
 template <int WIN>
-__device__ __forceinline__ float abs_residual(const Level &L, float qx, float qy, int lane,
-                                              const float (&T)[KRuns<WIN>::NS], KSmem<WIN> &sm) {
-    constexpr int HW = WIN / 2, JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
-    const float fx = floorf(qx), fy = floorf(qy);
-    const float bx = qx - fx, by = qy - fy;
-    const int off = stage_footprint<WIN>(L, (int)fx - HW, (int)fy - HW, lane, sm);
+__device__ __forceinline__ float abs_residual(const KCta<WIN> &C, int x0, int w, float bx, float by, int lane,
+                                              const float (&T)[KRuns<WIN>::NS], const KSmem<WIN> &sm) {
+    constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     float sa = 0.f, sb = 0.f;
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
         int c, r0;
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
-        const uint8_t *jr = valid ? &sm.j[r0 * JS + off + c] : sm.zj;
+        int o0, o1;
+        run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
+        const uint8_t *j0 = valid ? &sm.j[r0 * JS + o0] : C.zj, *j1 = valid ? &sm.j[r0 * JS + o1] : C.zj;
         float ph = 0.f;
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(jr[r * JS]);
-            const float h = fmaf(bx, u8f(jr[r * JS + 1]) - mv, mv);
+            const float mv = u8f(j0[r * JS]);
+            const float h = fmaf(bx, u8f(j1[r * JS]) - mv, mv);
             if (r > 0) {
                 const float jv = fmaf(by, h - ph, ph);
                 const float e = fabsf(T[i * RL + r - 1] - jv);  // 0 - 0 for a run outside the window
@@ -506,7 +516,7 @@ __device__ __forceinline__ float abs_residual(const Level &L, float qx, float qy
 // G and b lose the weak direction: their rounding, divided by lambda_min,
 // moves the Newton steps along it by more than the flow tolerance.  Such a
 // level is tracked in FP64: the template and its gradients are sampled in
-// FP64 from the staged windows (kept in sm.t / sm.g) at every sweep, G, the
+// FP64 from the level's staged windows at every sweep, G, the
 // footprint moments, the 2x2 solve and the position update are FP64.  The
 // branch is warp-uniform; with the default eigenvalue threshold (1e-4) an
 // accepted template cannot exceed a condition number of 5e3 (fp64_needed),
@@ -518,29 +528,18 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Keep the template's image window: copy sm.j (as staged by load_template)
-// to sm.t before footprints overwrite it.
-template <int WIN>
-__device__ __forceinline__ void keep_template_window(int lane, KSmem<WIN> &sm) {
-    constexpr int NB = (WIN + 1) * KSmem<WIN>::JS / 16;
-    __syncwarp();
-    const uint4 *src = reinterpret_cast<const uint4 *>(sm.j);
-    uint4 *dst = reinterpret_cast<uint4 *>(sm.t);
-    for (int k = lane; k < NB; k += 32) dst[k] = src[k];
-    __syncwarp();
-}
-
 // The lane's samples of one staged template row pair in FP64: horizontal
-// lerps of row r of the template image and gradient windows.
+// lerps of row r of the template image and gradient windows (d: the right
+// neighbour's distance, 0 where it is clamped).
 template <int WIN, int GT>
-__device__ __forceinline__ void tmpl_row64(const uint8_t *tr, const uint32_t *gr, int r, double ax, double unit,
+__device__ __forceinline__ void tmpl_row64(const uint8_t *tr, const uint32_t *gr, int d, int r, double ax, double unit,
                                            double &hT, double &hGX, double &hGY) {
     constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS;
     constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
-    const double t0 = (double)tr[r * JS], t1 = (double)tr[r * JS + 1];
+    const double t0 = (double)tr[r * JS], t1 = (double)tr[r * JS + d];
     float gx0, gy0, gx1, gy1;
     unpack_grad<GTS>(gr[r * GS], gx0, gy0);
-    unpack_grad<GTS>(gr[r * GS + 1], gx1, gy1);
+    unpack_grad<GTS>(gr[r * GS + d], gx1, gy1);
     const double x0 = (double)gx0 * unit, x1 = (double)gx1 * unit, y0 = (double)gy0 * unit, y1 = (double)gy1 * unit;
     hT = fma(ax, t1 - t0, t0);
     hGX = fma(ax, x1 - x0, x0);
@@ -550,8 +549,8 @@ __device__ __forceinline__ void tmpl_row64(const uint8_t *tr, const uint32_t *gr
 // G of the level's template in FP64 (grey levels per pixel), every lane
 // holding the totals.
 template <int WIN, int GT>
-__device__ __forceinline__ void template_G64(double ax, double ay, int offi, int offg, int lane, const KSmem<WIN> &sm,
-                                             double &g11, double &g12, double &g22) {
+__device__ __forceinline__ void template_G64(double ax, double ay, int tx0, int tw, int lane, const uint8_t *st,
+                                             const uint32_t *sg, double &g11, double &g12, double &g22) {
     constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     constexpr double unit = (double)grad_unit<GT>();
     double a11 = 0.0, a12 = 0.0, a22 = 0.0;
@@ -561,14 +560,16 @@ __device__ __forceinline__ void template_G64(double ax, double ay, int offi, int
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
         if (!valid) continue;
-        const uint8_t *tr = &sm.t[r0 * JS + offi + c];
-        const uint32_t *gr = &sm.g[r0 * GS + offg + c];
+        int t0, t1;
+        run_columns<WIN>(tx0, tw, staged_x(tx0, 16), c, t0, t1);
+        const uint8_t *tr = st + r0 * JS + t0;
+        const uint32_t *gr = sg + r0 * GS + t0 + staged_x(tx0, 16) - staged_x(tx0, 4);
         double pT, pX, pY;
-        tmpl_row64<WIN, GT>(tr, gr, 0, ax, unit, pT, pX, pY);
+        tmpl_row64<WIN, GT>(tr, gr, t1 - t0, 0, ax, unit, pT, pX, pY);
 #pragma unroll 1
         for (int r = 1; r <= RL; ++r) {
             double hT, hX, hY;
-            tmpl_row64<WIN, GT>(tr, gr, r, ax, unit, hT, hX, hY);
+            tmpl_row64<WIN, GT>(tr, gr, t1 - t0, r, ax, unit, hT, hX, hY);
             const double gx = fma(ay, hX - pX, pX), gy = fma(ay, hY - pY, pY);
             a11 = fma(gx, gx, a11);
             a12 = fma(gx, gy, a12);
@@ -584,13 +585,14 @@ __device__ __forceinline__ void template_G64(double ax, double ay, int offi, int
 }
 
 // The eight footprint moments of cell_moments in FP64, the template sampled
-// in FP64 from the kept windows (grey levels per pixel).
+// in FP64 from its staged windows (grey levels per pixel).
 template <int WIN, int GT>
-__device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, double ax, double ay, int offi,
-                                               int offg, int lane, KSmem<WIN> &sm, double (&m)[8]) {
+__device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, double ax, double ay, int tx0,
+                                               int tw, int lane, const uint8_t *st, const uint32_t *sg,
+                                               KSmem<WIN> &sm, double (&m)[8]) {
     constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     constexpr double unit = (double)grad_unit<GT>();
-    const int off = stage_footprint<WIN>(L, x0, y0, lane, sm);
+    stage_footprint<WIN>(L, x0, y0, lane, sm);
     double a[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) a[k] = 0.0;
@@ -600,20 +602,24 @@ __device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, d
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
         if (!valid) continue;
-        const uint8_t *tr = &sm.t[r0 * JS + offi + c];
-        const uint32_t *gr = &sm.g[r0 * GS + offg + c];
-        const uint8_t *jr = &sm.j[r0 * JS + off + c];
+        int t0, t1;
+        run_columns<WIN>(tx0, tw, staged_x(tx0, 16), c, t0, t1);
+        const uint8_t *tr = st + r0 * JS + t0;
+        const uint32_t *gr = sg + r0 * GS + t0 + staged_x(tx0, 16) - staged_x(tx0, 4);
+        int o0, o1;
+        run_columns<WIN>(x0, L.w, staged_x(x0, 16), c, o0, o1);
+        const uint8_t *j0 = &sm.j[r0 * JS + o0], *j1 = &sm.j[r0 * JS + o1];
         double pT, pX, pY;
-        tmpl_row64<WIN, GT>(tr, gr, 0, ax, unit, pT, pX, pY);
-        double pmv = (double)jr[0];
-        double pdx = (double)jr[1] - pmv;
+        tmpl_row64<WIN, GT>(tr, gr, t1 - t0, 0, ax, unit, pT, pX, pY);
+        double pmv = (double)j0[0];
+        double pdx = (double)j1[0] - pmv;
 #pragma unroll 1
         for (int r = 1; r <= RL; ++r) {
             double hT, hX, hY;
-            tmpl_row64<WIN, GT>(tr, gr, r, ax, unit, hT, hX, hY);
+            tmpl_row64<WIN, GT>(tr, gr, t1 - t0, r, ax, unit, hT, hX, hY);
             const double T = fma(ay, hT - pT, pT), gx = fma(ay, hX - pX, pX), gy = fma(ay, hY - pY, pY);
-            const double mv = (double)jr[r * JS];
-            const double dx = (double)jr[r * JS + 1] - mv;
+            const double mv = (double)j0[r * JS];
+            const double dx = (double)j1[r * JS] - mv;
             const double e0 = T - pmv, sy = mv - pmv, sxy = dx - pdx;
             a[0] = fma(e0, gx, a[0]);
             a[1] = fma(pdx, gx, a[1]);
@@ -646,8 +652,9 @@ struct Level64 {
 // iterations from the level's guess (gx, gy).
 template <int WIN, int GT>
 __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_iters, const float eps2,
-                                              const float min_eig, float ux, float uy, float gx, float gy, int offi,
-                                              int offg, int lane, KSmem<WIN> *smp) {
+                                              const float min_eig, float ux, float uy, float gx, float gy, int tx0,
+                                              int tw, int lane, const uint8_t *st, const uint32_t *sg,
+                                              KSmem<WIN> *smp) {
     constexpr int HW = WIN / 2;
     constexpr double N = (double)(WIN * WIN);
     KSmem<WIN> &sm = *smp;
@@ -656,10 +663,9 @@ __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_i
     o.iters = 0;
     o.sweeps = 0;
     o.nx = o.ny = 0.0;
-    keep_template_window<WIN>(lane, sm);
     const double ax = (double)(ux - floorf(ux)), ay = (double)(uy - floorf(uy));
     double G11, G12, G22;
-    template_G64<WIN, GT>(ax, ay, offi, offg, lane, sm, G11, G12, G22);
+    template_G64<WIN, GT>(ax, ay, tx0, tw, lane, st, sg, G11, G12, G22);
     const double det64 = G11 * G22 - G12 * G12;
     const double lmax64 = 0.5 * (G11 + G22 + sqrt((G11 - G22) * (G11 - G22) + 4.0 * G12 * G12));
     const double lmin64 = det64 / lmax64 / (N * 65025.0);
@@ -682,7 +688,7 @@ __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_i
         const double fx = floor(qx), fy = floor(qy);
         const int ix = (int)fx - HW, iy = (int)fy - HW;
         if (ix != cx || iy != cy) {
-            cell_moments64<WIN, GT>(Jl, ix, iy, ax, ay, offi, offg, lane, sm, m);
+            cell_moments64<WIN, GT>(Jl, ix, iy, ax, ay, tx0, tw, lane, st, sg, sm, m);
             cx = ix;
             cy = iy;
             ++o.sweeps;
@@ -714,8 +720,8 @@ constexpr uint8_t kStatusPending = 2;
 // code out of the FP32 kernels keeps their registers free of it.
 template <int WIN, int GT, bool F64>
 __device__ __forceinline__ void track_point(const Level *I, const Level *J, const KParams &P, float ux0, float uy0,
-                                            bool has_guess, float gux, float guy, int lane, KSmem<WIN> &sm, KOut &o,
-                                            bool want_err) {
+                                            bool has_guess, float gux, float guy, int lane, const KCta<WIN> &C,
+                                            KSmem<WIN> &sm, KOut &o, bool want_err) {
     constexpr int HW = WIN / 2;
     constexpr float N = (float)(WIN * WIN);
     constexpr float unit = grad_unit<GT>();
@@ -748,14 +754,51 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         gx = (gux - ux0) * s;
         gy = (guy - uy0) * s;
     }
-    for (int l = L - 1; l >= 0; --l) {
-        // by value: the fields stay in registers across the staging copies
-        const Level Il = I[l];
-        const Level Jl = J[l];
-        const float s = pow2neg(l);
-        const float ux = ux0 * s, uy = uy0 * s;
-        int offi, offg;
-        load_template<WIN, GT>(Il, ux, uy, lane, T, GX, GY, sm, offi, offg);
+    int cx = INT_MIN, cy = INT_MIN;  // footprint cell last staged in sm.j (unknown: INT_MIN)
+    // Level l's iteration starts its own first footprint (its position is known
+    // now) and the next level's template (known from the start) before it
+    // samples its own template, which the previous iteration started: the
+    // copies arrive while the warp computes.  l = L only starts the first
+    // template.  Two commit groups per level, so the waits below count them.
+    for (int l = L; l >= 0; --l) {
+        float ux = 0.f, uy = 0.f;
+        Level Jl;
+        cx = INT_MIN;
+        if (l < L) {
+            Jl = J[l];  // by value: the fields stay in registers across the copies
+            const float s = pow2neg(l);
+            ux = ux0 * s, uy = uy0 * s;
+            const float qx = ux + gx, qy = uy + gy;
+            const float dist = fminf(fminf(qx + (float)HW, (float)(Jl.w - 1 + HW) - qx),
+                                     fminf(qy + (float)HW, (float)(Jl.h - 1 + HW) - qy));
+            if (dist >= 0.f) {
+                cx = (int)floorf(qx) - HW;
+                cy = (int)floorf(qy) - HW;
+                stage_window<WIN, false>(Jl, cx, cy, lane, sm.j, nullptr);
+            }
+            cp_async_commit();
+        }
+        if (GT != VT_GRAD_NONE && l > 0) {
+            const Level In = I[l - 1];
+            const float s = pow2neg(l - 1);
+            stage_window<WIN, true>(In, (int)floorf(ux0 * s) - HW, (int)floorf(uy0 * s) - HW, lane, sm.t[(l - 1) & 1],
+                                    sm.g[(l - 1) & 1]);
+        }
+        cp_async_commit();
+        if (l == L) continue;
+        uint8_t *st = sm.t[l & 1];
+        uint32_t *sg = sm.g[l & 1];
+        const float ax = ux - floorf(ux), ay = uy - floorf(uy);
+        int tx0 = (int)floorf(ux) - HW, tw = I[l].w;  // leftmost template column, level width
+        if constexpr (GT == VT_GRAD_NONE) {
+            __syncwarp();
+            stage_window_otf<WIN>(I[l], tx0, (int)floorf(uy) - HW, lane, st, sg);
+            tx0 = 0, tw = WIN + 1;  // staged column by column from 0, clamped already
+        } else {
+            cp_async_wait<2>();
+            __syncwarp();
+        }
+        sample_template<WIN, GT>(C, st, sg, tx0, tw, ax, ay, lane, T, GX, GY);
         ++o.tmpl;
         float a11 = 0.f, a12 = 0.f, a22 = 0.f;
 #pragma unroll
@@ -777,12 +820,15 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         level64 = P.fp64 && !(lmin * kFp64Cond >= lmax);
         if (level64) {
             if constexpr (!F64) {
+                cp_async_wait<0>();  // nothing may land after the buffers are used again
                 o.status = 0;
                 o.reason = kReasonPending;
                 return;
             } else {
-                const Level64 r = track_level64<WIN, GT>(Jl, P.max_iters, P.eps2, P.min_eig, ux, uy, gx, gy, offi,
-                                                         offg, lane, &sm);
+                cp_async_wait<0>();  // the first footprint started above: sm.j is staged anew
+                const Level64 r = track_level64<WIN, GT>(Jl, P.max_iters, P.eps2, P.min_eig, ux, uy, gx, gy, tx0,
+                                                         tw, lane, st, sg, &sm);
+                cx = INT_MIN;
                 o.lmin = r.lmin;
                 o.iters += r.iters;
                 o.sweeps += r.sweeps;
@@ -813,9 +859,11 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         // products cancel for ill-conditioned G, hence kdiff)
         const float inv_det = 1.0f / (det * unit);
         // moments of the footprint cell last swept (valid while the integer
-        // part of q does not change)
-        int cx = INT_MIN, cy = INT_MIN;
+        // part of q does not change); the first cell's copy was started above
         float m[8];
+        bool swept = false;
+        cp_async_wait<1>();
+        __syncwarp();
         for (int k = 0; k < P.max_iters; ++k) {
             const float qx = ux + gx + nux, qy = uy + gy + nuy;
             const float dist = fminf(fminf(qx + (float)HW, (float)(Jl.w - 1 + HW) - qx),
@@ -827,8 +875,10 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             }
             const float fx = floorf(qx), fy = floorf(qy);
             const int ix = (int)fx - HW, iy = (int)fy - HW;
-            if (ix != cx || iy != cy) {
-                cell_moments<WIN>(Jl, ix, iy, lane, T, GX, GY, sm, m);
+            if (!swept || ix != cx || iy != cy) {
+                if (ix != cx || iy != cy) stage_footprint<WIN>(Jl, ix, iy, lane, sm);
+                cell_moments<WIN>(ix, Jl.w, lane, T, GX, GY, sm, m);
+                swept = true;
                 cx = ix;
                 cy = iy;
                 ++o.sweeps;
@@ -852,6 +902,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             gy = 2.f * (gy + nuy);
         }
     }
+    cp_async_wait<0>();  // a point lost early leaves copies under way; nothing may land after this
     {
         const float sc = (float)(1 << lost_level);
         const float si = pow2neg(lost_level);
@@ -869,9 +920,12 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             o.status = 0;
             o.reason = VT_LOST_OOB;
         } else {
-            // T still holds level 0's template
+            // T still holds level 0's template, and sm.j its last footprint
             if (want_err) {
-                o.err = abs_residual<WIN>(J[0], o.x, o.y, lane, T, sm) / N;
+                const float fx = floorf(o.x), fy = floorf(o.y);
+                const int ix = (int)fx - HW, iy = (int)fy - HW;
+                if (ix != cx || iy != cy) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
+                o.err = abs_residual<WIN>(C, ix, J[0].w, o.x - fx, o.y - fy, lane, T, sm) / N;
                 ++o.errp;
             }
         }
@@ -885,7 +939,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
 template <int WIN, int GT, bool F64>
 __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, const KParams &P, float ux0,
                                                 float uy0, bool fb, bool has_guess, float gux, float guy, int lane,
-                                                KSmem<WIN> &sm, KOut &o) {
+                                                const KCta<WIN> &C, KSmem<WIN> &sm, KOut &o) {
     const Level *A = I, *B = J;
     float x = ux0, y = uy0;
     const int npass = fb ? 2 : 1;
@@ -893,7 +947,7 @@ __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, 
     for (int pass = 0; pass < npass; ++pass) {
         KOut r;
         // the backward pass only decides the status: its error is not an output
-        track_point<WIN, GT, F64>(A, B, P, x, y, pass == 0 && has_guess, gux, guy, lane, sm, r, pass == 0);
+        track_point<WIN, GT, F64>(A, B, P, x, y, pass == 0 && has_guess, gux, guy, lane, C, sm, r, pass == 0);
         if (pass == 0) {
             o = r;
             if (!r.status) return;
