@@ -122,6 +122,12 @@ __device__ __forceinline__ void warp_sum3(float x, float y, float z, int lane, f
 // conversion would load.
 __device__ __forceinline__ float u8f(uint32_t v) { return __uint2float_rn(v); }
 
+// Packed FP32 pairs: this GPU issues one instruction for two FMAs, each
+// rounded as the scalar one.  y - x as x * (-1) + y: the product is exact, so
+// the result is the subtraction's.
+__device__ __forceinline__ float2 pair(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 y, float2 x) { return __ffma2_rn(x, pair(-1.f), y); }
+
 template <int GT>
 __device__ __forceinline__ void unpack_grad(uint32_t v, float &gx, float &gy) {
     if (GT == VT_GRAD_S16) {
@@ -386,7 +392,7 @@ __device__ __forceinline__ void run_columns(int x0, int w, int sx, int c, int &o
 template <int WIN, int GT>
 __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_t *st, const uint32_t *sg, int x0,
                                                 int w, float ax, float ay, int lane, float (&T)[KRuns<WIN>::NS],
-                                                float (&GX)[KRuns<WIN>::NS], float (&GY)[KRuns<WIN>::NS]) {
+                                                float2 (&G)[KRuns<WIN>::NS]) {
     constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     // staged gradient words are int16 pairs when computed in place
     constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
@@ -400,24 +406,22 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_
         const uint8_t *j0 = valid ? st + r0 * JS + o0 : C.zj, *j1 = valid ? st + r0 * JS + o1 : C.zj;
         const int dg = staged_x(x0, 16) - staged_x(x0, 4);
         const uint32_t *g0 = valid ? sg + r0 * GS + o0 + dg : C.zg, *g1 = valid ? sg + r0 * GS + o1 + dg : C.zg;
-        float pi = 0.f, pgx = 0.f, pgy = 0.f;
+        float pi = 0.f;
+        float2 pg = pair(0.f);
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
             const float mv = u8f(j0[r * JS]), mvr = u8f(j1[r * JS]);
-            float gx, gy, gxr, gyr;
-            unpack_grad<GTS>(g0[r * GS], gx, gy);
-            unpack_grad<GTS>(g1[r * GS], gxr, gyr);
+            float2 gl, gr;
+            unpack_grad<GTS>(g0[r * GS], gl.x, gl.y);
+            unpack_grad<GTS>(g1[r * GS], gr.x, gr.y);
             const float hi = fmaf(ax, mvr - mv, mv);
-            const float hgx = fmaf(ax, gxr - gx, gx);
-            const float hgy = fmaf(ax, gyr - gy, gy);
+            const float2 hg = __ffma2_rn(pair(ax), sub2(gr, gl), gl);
             if (r > 0) {
                 T[i * RL + r - 1] = fmaf(ay, hi - pi, pi);  // zero for a run outside the window
-                GX[i * RL + r - 1] = fmaf(ay, hgx - pgx, pgx);
-                GY[i * RL + r - 1] = fmaf(ay, hgy - pgy, pgy);
+                G[i * RL + r - 1] = __ffma2_rn(pair(ay), sub2(hg, pg), pg);
             }
             pi = hi;
-            pgx = hgx;
-            pgy = hgy;
+            pg = hg;
         }
     }
 }
@@ -435,12 +439,12 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_
 // in sm.j; w: the level's width.
 template <int WIN>
 __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&T)[KRuns<WIN>::NS],
-                                             const float (&GX)[KRuns<WIN>::NS], const float (&GY)[KRuns<WIN>::NS],
-                                             const KSmem<WIN> &sm, float (&m)[8]) {
+                                             const float2 (&G)[KRuns<WIN>::NS], const KSmem<WIN> &sm,
+                                             float (&m)[8]) {
     constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
-    float a[8];
+    float2 a[4];  // (x part, y part) of each moment
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = 0.f;
+    for (int k = 0; k < 4; ++k) a[k] = pair(0.f);
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
         int c, r0;
@@ -449,31 +453,26 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
         int o0, o1;
         run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
         const uint8_t *j0 = &sm.j[r0 * JS + o0], *j1 = &sm.j[r0 * JS + o1];
-        float pmv = 0.f, pdx = 0.f;
+        float2 p = pair(0.f);  // F and F(c + 1) - F(c) of the row above
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(j0[r * JS]);
-            const float dx = u8f(j1[r * JS]) - mv;  // F(r, c+1) - F(r, c), exact
+            float2 q;
+            q.x = u8f(j0[r * JS]);
+            q.y = u8f(j1[r * JS]) - q.x;  // exact
             if (r > 0) {
                 const int s = i * RL + r - 1;
-                const float e0 = T[s] - pmv;
-                const float sy = mv - pmv;   // F10 - F00
-                const float sxy = dx - pdx;  // F11 - F10 - F01 + F00
-                const float gx = GX[s], gy = GY[s];
-                a[0] = fmaf(e0, gx, a[0]);
-                a[1] = fmaf(pdx, gx, a[1]);
-                a[2] = fmaf(sy, gx, a[2]);
-                a[3] = fmaf(sxy, gx, a[3]);
-                a[4] = fmaf(e0, gy, a[4]);
-                a[5] = fmaf(pdx, gy, a[5]);
-                a[6] = fmaf(sy, gy, a[6]);
-                a[7] = fmaf(sxy, gy, a[7]);
+                const float e0 = T[s] - p.x;
+                const float2 d = sub2(q, p);  // F10 - F00, F11 - F10 - F01 + F00
+                a[0] = __ffma2_rn(pair(e0), G[s], a[0]);
+                a[1] = __ffma2_rn(pair(p.y), G[s], a[1]);
+                a[2] = __ffma2_rn(pair(d.x), G[s], a[2]);
+                a[3] = __ffma2_rn(pair(d.y), G[s], a[3]);
             }
-            pmv = mv;
-            pdx = dx;
+            p = q;
         }
     }
-    warp_sum8(a, lane, m);
+    const float v[8] = {a[0].x, a[1].x, a[2].x, a[3].x, a[0].y, a[1].y, a[2].y, a[3].y};
+    warp_sum8(v, lane, m);
 }
 
 // Error sweep over the staged footprint at fractional offset (bx, by): sum
@@ -728,7 +727,8 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
     // lambda_min normalisation: stored units^2 -> (grey/px)^2, / (N 255^2)
     const float inv_norm = unit * unit / (N * 65025.0f);
     constexpr int NS = KRuns<WIN>::NS;
-    float T[NS], GX[NS], GY[NS];
+    float T[NS];
+    float2 G[NS];
     const int L = P.levels;
     float gx = 0.f, gy = 0.f, nux = 0.f, nuy = 0.f;
     double nx64 = 0.0, ny64 = 0.0;  // the step sum of an FP64 level
@@ -798,17 +798,17 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             cp_async_wait<2>();
             __syncwarp();
         }
-        sample_template<WIN, GT>(C, st, sg, tx0, tw, ax, ay, lane, T, GX, GY);
+        sample_template<WIN, GT>(C, st, sg, tx0, tw, ax, ay, lane, T, G);
         ++o.tmpl;
-        float a11 = 0.f, a12 = 0.f, a22 = 0.f;
+        float2 aii = pair(0.f);
+        float a12 = 0.f;
 #pragma unroll
         for (int r = 0; r < NS; ++r) {
-            a11 = fmaf(GX[r], GX[r], a11);
-            a12 = fmaf(GX[r], GY[r], a12);
-            a22 = fmaf(GY[r], GY[r], a22);
+            aii = __ffma2_rn(G[r], G[r], aii);
+            a12 = fmaf(G[r].x, G[r].y, a12);
         }
         float g11, g12, g22;
-        warp_sum3(a11, a12, a22, lane, g11, g12, g22);
+        warp_sum3(aii.x, a12, aii.y, lane, g11, g12, g22);
         // lambda_min = det / lambda_max avoids the cancellation of (tr - disc) / 2
         const float tr = g11 + g22, df = g11 - g22;
         const float lmax = 0.5f * (tr + sqrtf(fmaf(df, df, 4.f * g12 * g12)));
@@ -877,7 +877,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             const int ix = (int)fx - HW, iy = (int)fy - HW;
             if (!swept || ix != cx || iy != cy) {
                 if (ix != cx || iy != cy) stage_footprint<WIN>(Jl, ix, iy, lane, sm);
-                cell_moments<WIN>(ix, Jl.w, lane, T, GX, GY, sm, m);
+                cell_moments<WIN>(ix, Jl.w, lane, T, G, sm, m);
                 swept = true;
                 cx = ix;
                 cy = iy;
