@@ -434,13 +434,13 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_
 //   sum r grad T = R - bx Sx - by Sy - bx by Sxy,
 //   R = sum (T - F00) grad T, Sx = sum (F01 - F00) grad T,
 //   Sy = sum (F10 - F00) grad T, Sxy = sum (F11 - F10 - F01 + F00) grad T.
-// The footprint differences are exact (integers); m[0..3] are the x parts
-// (R, Sx, Sy, Sxy against Tx), m[4..7] the y parts.  The footprint is staged
+// The footprint differences are exact (integers); m: R, Sx, Sy, Sxy as (x
+// part, y part).  The footprint is staged
 // in sm.j; w: the level's width.
 template <int WIN>
 __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&T)[KRuns<WIN>::NS],
                                              const float2 (&G)[KRuns<WIN>::NS], const KSmem<WIN> &sm,
-                                             float (&m)[8]) {
+                                             float2 (&m)[4]) {
     constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     float2 a[4];  // (x part, y part) of each moment
 #pragma unroll
@@ -472,7 +472,10 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
         }
     }
     const float v[8] = {a[0].x, a[1].x, a[2].x, a[3].x, a[0].y, a[1].y, a[2].y, a[3].y};
-    warp_sum8(v, lane, m);
+    float t[8];
+    warp_sum8(v, lane, t);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = make_float2(t[k], t[k + 4]);
 }
 
 // Error sweep over the staged footprint at fractional offset (bx, by): sum
@@ -754,51 +757,62 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         gx = (gux - ux0) * s;
         gy = (guy - uy0) * s;
     }
-    int cx = INT_MIN, cy = INT_MIN;  // footprint cell last staged in sm.j (unknown: INT_MIN)
+    // integer part of the footprint position last staged in sm.j (unknown: NaN)
+    constexpr float kNone = __builtin_nanf("");
+    float cfx = kNone, cfy = kNone;
+    // the template started by the previous iteration: position, its floor, the level's width
+    float ux = 0.f, uy = 0.f, ufx = 0.f, ufy = 0.f;
+    int tw = 0;
+    float s = pow2neg(L);
     // Level l's iteration starts its own first footprint (its position is known
     // now) and the next level's template (known from the start) before it
     // samples its own template, which the previous iteration started: the
     // copies arrive while the warp computes.  l = L only starts the first
     // template.  Two commit groups per level, so the waits below count them.
     for (int l = L; l >= 0; --l) {
-        float ux = 0.f, uy = 0.f;
+        const float ax = ux - ufx, ay = uy - ufy;
+        int tx0 = (int)ufx - HW;  // leftmost template column
+        const int ty0 = (int)ufy - HW, w_I = tw;
+        const float qx0 = ux + gx, qy0 = uy + gy;  // the level's first footprint position
+        float limx = 0.f, limy = 0.f;              // footprint positions lie in [-HW, limx] x [-HW, limy]
+        bool inside = false;
         Level Jl;
-        cx = INT_MIN;
+        cfx = kNone;
         if (l < L) {
             Jl = J[l];  // by value: the fields stay in registers across the copies
-            const float s = pow2neg(l);
-            ux = ux0 * s, uy = uy0 * s;
-            const float qx = ux + gx, qy = uy + gy;
-            const float dist = fminf(fminf(qx + (float)HW, (float)(Jl.w - 1 + HW) - qx),
-                                     fminf(qy + (float)HW, (float)(Jl.h - 1 + HW) - qy));
-            if (dist >= 0.f) {
-                cx = (int)floorf(qx) - HW;
-                cy = (int)floorf(qy) - HW;
-                stage_window<WIN, false>(Jl, cx, cy, lane, sm.j, nullptr);
+            limx = (float)(Jl.w - 1 + HW);
+            limy = (float)(Jl.h - 1 + HW);
+            inside = qx0 >= -(float)HW && qx0 <= limx && qy0 >= -(float)HW && qy0 <= limy;
+            if (inside) {
+                cfx = floorf(qx0);
+                cfy = floorf(qy0);
+                stage_window<WIN, false>(Jl, (int)cfx - HW, (int)cfy - HW, lane, sm.j, nullptr);
             }
             cp_async_commit();
         }
-        if (GT != VT_GRAD_NONE && l > 0) {
+        if (l > 0) {
             const Level In = I[l - 1];
-            const float s = pow2neg(l - 1);
-            stage_window<WIN, true>(In, (int)floorf(ux0 * s) - HW, (int)floorf(uy0 * s) - HW, lane, sm.t[(l - 1) & 1],
-                                    sm.g[(l - 1) & 1]);
+            s += s;
+            ux = ux0 * s, uy = uy0 * s;
+            ufx = floorf(ux), ufy = floorf(uy);
+            tw = In.w;
+            if constexpr (GT != VT_GRAD_NONE)
+                stage_window<WIN, true>(In, (int)ufx - HW, (int)ufy - HW, lane, sm.t[(l - 1) & 1], sm.g[(l - 1) & 1]);
         }
         cp_async_commit();
         if (l == L) continue;
         uint8_t *st = sm.t[l & 1];
         uint32_t *sg = sm.g[l & 1];
-        const float ax = ux - floorf(ux), ay = uy - floorf(uy);
-        int tx0 = (int)floorf(ux) - HW, tw = I[l].w;  // leftmost template column, level width
         if constexpr (GT == VT_GRAD_NONE) {
             __syncwarp();
-            stage_window_otf<WIN>(I[l], tx0, (int)floorf(uy) - HW, lane, st, sg);
-            tx0 = 0, tw = WIN + 1;  // staged column by column from 0, clamped already
+            stage_window_otf<WIN>(I[l], tx0, ty0, lane, st, sg);
+            tx0 = 0;  // staged column by column from 0, clamped already
+            sample_template<WIN, GT>(C, st, sg, 0, WIN + 1, ax, ay, lane, T, G);
         } else {
             cp_async_wait<2>();
             __syncwarp();
+            sample_template<WIN, GT>(C, st, sg, tx0, w_I, ax, ay, lane, T, G);
         }
-        sample_template<WIN, GT>(C, st, sg, tx0, tw, ax, ay, lane, T, G);
         ++o.tmpl;
         float2 aii = pair(0.f);
         float a12 = 0.f;
@@ -826,9 +840,10 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
                 return;
             } else {
                 cp_async_wait<0>();  // the first footprint started above: sm.j is staged anew
-                const Level64 r = track_level64<WIN, GT>(Jl, P.max_iters, P.eps2, P.min_eig, ux, uy, gx, gy, tx0,
-                                                         tw, lane, st, sg, &sm);
-                cx = INT_MIN;
+                const Level64 r = track_level64<WIN, GT>(Jl, P.max_iters, P.eps2, P.min_eig, ux0 * pow2neg(l),
+                                                         uy0 * pow2neg(l), gx, gy, tx0,
+                                                         GT == VT_GRAD_NONE ? WIN + 1 : w_I, lane, st, sg, &sm);
+                cfx = kNone;
                 o.lmin = r.lmin;
                 o.iters += r.iters;
                 o.sweeps += r.sweeps;
@@ -858,40 +873,55 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         // (unit is a power of two, so det * unit is exact; the adjugate
         // products cancel for ill-conditioned G, hence kdiff)
         const float inv_det = 1.0f / (det * unit);
-        // moments of the footprint cell last swept (valid while the integer
-        // part of q does not change); the first cell's copy was started above
-        float m[8];
-        bool swept = false;
+        if (!inside) {
+            o.status = 0;
+            o.reason = VT_LOST_OOB;
+            lost_level = l;
+            break;
+        }
+        // the moments of a footprint cell serve every position in it; the
+        // first cell's copy was started above
+        float2 m[4];
         cp_async_wait<1>();
         __syncwarp();
-        for (int k = 0; k < P.max_iters; ++k) {
-            const float qx = ux + gx + nux, qy = uy + gy + nuy;
-            const float dist = fminf(fminf(qx + (float)HW, (float)(Jl.w - 1 + HW) - qx),
-                                     fminf(qy + (float)HW, (float)(Jl.h - 1 + HW) - qy));
-            if (!(dist >= 0.f)) {
-                o.status = 0;
-                o.reason = VT_LOST_OOB;
-                break;
-            }
-            const float fx = floorf(qx), fy = floorf(qy);
-            const int ix = (int)fx - HW, iy = (int)fy - HW;
-            if (!swept || ix != cx || iy != cy) {
-                if (ix != cx || iy != cy) stage_footprint<WIN>(Jl, ix, iy, lane, sm);
-                cell_moments<WIN>(ix, Jl.w, lane, T, G, sm, m);
-                swept = true;
-                cx = ix;
-                cy = iy;
-                ++o.sweeps;
-            }
-            const float bx = qx - fx, by = qy - fy, bxy = bx * by;
-            const float b1 = m[0] - bx * m[1] - by * m[2] - bxy * m[3];
-            const float b2 = m[4] - bx * m[5] - by * m[6] - bxy * m[7];
-            const float ex = kdiff(g22, b1, g12, b2) * inv_det;
-            const float ey = kdiff(g11, b2, g12, b1) * inv_det;
+        cell_moments<WIN>((int)cfx - HW, Jl.w, lane, T, G, sm, m);
+        ++o.sweeps;
+        float bx = qx0 - cfx, by = qy0 - cfy;
+        // A position is in the cell when both offsets lie in [0, 1): as bit
+        // patterns, below that of 1 (negative numbers and NaN are above).  A
+        // cell that begins at the bound holds positions outside: there every
+        // step takes the full test (0).
+        constexpr unsigned kOne = 0x3f800000u;
+        unsigned cell_end = cfx >= limx || cfy >= limy ? 0u : kOne;
+        for (int k = 1;; ++k) {
+            const float bxy = bx * by;
+            float2 b = __ffma2_rn(pair(-bx), m[1], m[0]);
+            b = __ffma2_rn(pair(-by), m[2], b);
+            b = __ffma2_rn(pair(-bxy), m[3], b);
+            const float ex = kdiff(g22, b.x, g12, b.y) * inv_det;
+            const float ey = kdiff(g11, b.y, g12, b.x) * inv_det;
             nux += ex;
             nuy += ey;
             ++o.iters;
-            if (ex * ex + ey * ey < P.eps2) break;
+            if (ex * ex + ey * ey < P.eps2 || k >= P.max_iters) break;
+            const float qx = qx0 + nux, qy = qy0 + nuy;
+            bx = qx - cfx, by = qy - cfy;
+            if (max(__float_as_uint(bx), __float_as_uint(by)) >= cell_end) {
+                if (!(qx >= -(float)HW && qx <= limx && qy >= -(float)HW && qy <= limy)) {
+                    o.status = 0;
+                    o.reason = VT_LOST_OOB;
+                    break;
+                }
+                const float fx = floorf(qx), fy = floorf(qy);
+                if (fx != cfx || fy != cfy) {
+                    cfx = fx, cfy = fy;
+                    stage_footprint<WIN>(Jl, (int)fx - HW, (int)fy - HW, lane, sm);
+                    cell_moments<WIN>((int)fx - HW, Jl.w, lane, T, G, sm, m);
+                    ++o.sweeps;
+                    bx = qx - fx, by = qy - fy;
+                    cell_end = fx >= limx || fy >= limy ? 0u : kOne;
+                }
+            }
         }
         if (!o.status) {
             lost_level = l;
@@ -924,7 +954,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             if (want_err) {
                 const float fx = floorf(o.x), fy = floorf(o.y);
                 const int ix = (int)fx - HW, iy = (int)fy - HW;
-                if (ix != cx || iy != cy) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
+                if (fx != cfx || fy != cfy) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
                 o.err = abs_residual<WIN>(C, ix, J[0].w, o.x - fx, o.y - fy, lane, T, sm) / N;
                 ++o.errp;
             }
