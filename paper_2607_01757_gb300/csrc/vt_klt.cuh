@@ -117,10 +117,18 @@ __device__ __forceinline__ void warp_sum3(float x, float y, float z, int lane, f
     sz = __shfl_sync(kFull, d, 16);
 }
 
-// A byte as a float (exact; differences of two are exact integers).  The
-// conversion runs on its own pipe, off the integer pipe that an OR-with-2^23
-// conversion would load.
-__device__ __forceinline__ float u8f(uint32_t v) { return __uint2float_rn(v); }
+// Image values in the FP32 sweeps are kept times 2^-22: a byte's bit pattern
+// read as a float is the denormal byte * 2^-149, so one FP32 multiplication by
+// 2^127 (exact, full rate) converts it, and one FMA converts and subtracts.
+// The integer pipe, the busiest one, is left out (a conversion instruction
+// per byte kept it 7 % busier and cost an instruction more per pair of
+// neighbours).  A power of two changes no rounding: every result is the
+// unscaled one's, scaled, until kImgUnscale takes it back.
+constexpr float kImgUnscale = 4194304.f;  // 2^22
+__device__ __forceinline__ float px_scale() { return __int_as_float(0x7f000000); }  // 2^127
+__device__ __forceinline__ float px(uint32_t v) { return __uint_as_float(v) * px_scale(); }
+// px(v) - a (a the px of another byte: the difference is exact)
+__device__ __forceinline__ float px_minus(uint32_t v, float a) { return fmaf(__uint_as_float(v), px_scale(), -a); }
 
 // Packed FP32 pairs: this GPU issues one instruction for two FMAs, each
 // rounded as the scalar one.  y - x as x * (-1) + y: the product is exact, so
@@ -386,7 +394,7 @@ __device__ __forceinline__ void run_columns(int x0, int w, int sx, int c, int &o
     }
 }
 
-// The template at the lane's window samples (KRuns): T and its gradients,
+// The template at the lane's window samples (KRuns): T (times 2^-22, see px) and its gradients,
 // sampled at fractional offset (ax, ay) from the staged windows, zero for
 // samples outside the window.
 template <int WIN, int GT>
@@ -410,11 +418,11 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_
         float2 pg = pair(0.f);
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(j0[r * JS]), mvr = u8f(j1[r * JS]);
+            const float mv = px(j0[r * JS]);
             float2 gl, gr;
             unpack_grad<GTS>(g0[r * GS], gl.x, gl.y);
             unpack_grad<GTS>(g1[r * GS], gr.x, gr.y);
-            const float hi = fmaf(ax, mvr - mv, mv);
+            const float hi = fmaf(ax, px_minus(j1[r * JS], mv), mv);
             const float2 hg = __ffma2_rn(pair(ax), sub2(gr, gl), gl);
             if (r > 0) {
                 T[i * RL + r - 1] = fmaf(ay, hi - pi, pi);  // zero for a run outside the window
@@ -457,8 +465,8 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
             float2 q;
-            q.x = u8f(j0[r * JS]);
-            q.y = u8f(j1[r * JS]) - q.x;  // exact
+            q.x = px(j0[r * JS]);
+            q.y = px_minus(j1[r * JS], q.x);
             if (r > 0) {
                 const int s = i * RL + r - 1;
                 const float e0 = T[s] - p.x;
@@ -496,8 +504,8 @@ __device__ __forceinline__ float abs_residual(const KCta<WIN> &C, int x0, int w,
         float ph = 0.f;
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = u8f(j0[r * JS]);
-            const float h = fmaf(bx, u8f(j1[r * JS]) - mv, mv);
+            const float mv = px(j0[r * JS]);
+            const float h = fmaf(bx, px_minus(j1[r * JS], mv), mv);
             if (r > 0) {
                 const float jv = fmaf(by, h - ph, ph);
                 const float e = fabsf(T[i * RL + r - 1] - jv);  // 0 - 0 for a run outside the window
@@ -872,7 +880,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         // eta = G^-1 b in grey/px units: G = unit^2 G_s, b = unit b_s => eta = adj(G_s) b_s / (unit det_s)
         // (unit is a power of two, so det * unit is exact; the adjugate
         // products cancel for ill-conditioned G, hence kdiff)
-        const float inv_det = 1.0f / (det * unit);
+        const float inv_det = 1.0f / (det * unit) * kImgUnscale;  // b carries the image scale
         if (!inside) {
             o.status = 0;
             o.reason = VT_LOST_OOB;
@@ -955,7 +963,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
                 const float fx = floorf(o.x), fy = floorf(o.y);
                 const int ix = (int)fx - HW, iy = (int)fy - HW;
                 if (fx != cfx || fy != cfy) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
-                o.err = abs_residual<WIN>(C, ix, J[0].w, o.x - fx, o.y - fy, lane, T, sm) / N;
+                o.err = abs_residual<WIN>(C, ix, J[0].w, o.x - fx, o.y - fy, lane, T, sm) * kImgUnscale / N;
                 ++o.errp;
             }
         }
