@@ -30,6 +30,7 @@
 #pragma once
 
 #include <climits>
+#include <cstddef>
 
 #include "vt_internal.cuh"
 
@@ -181,10 +182,36 @@ struct KSmem {
     static constexpr int NG = (4 * (3 + WIN + 1) + 15) / 16;  // 16-byte chunks per staged gradient row
     static constexpr int GS = NG * 4;                         // staged gradient row stride in words
     static_assert(GS >= 3 + WIN + 1, "a staged gradient row covers the window row");
+    Level lv[2][VT_MAX_LEVELS];  // the point's two pyramids
     uint8_t j[(WIN + 1) * JS];
-    uint8_t t[2][(WIN + 1) * JS];
     uint32_t g[2][(WIN + 1) * GS];
+    uint8_t t[2][(WIN + 1) * JS];
+    // Pyramids without gradient planes: the image windows of this level and the
+    // next, one pixel wider on every side, over g[1] and t; the gradients
+    // computed from them in g[0].
+    static constexpr int RS = (15 + WIN + 3 + 15) / 16 * 16, RAW = (WIN + 3) * RS;
+    __device__ __forceinline__ uint8_t *raw(int k) { return reinterpret_cast<uint8_t *>(g[1]) + k * RAW; }
 };
+template <int WIN>
+constexpr bool raw_fits() {
+    return 2 * KSmem<WIN>::RAW <= (int)(sizeof(KSmem<WIN>::g) / 2 + sizeof(KSmem<WIN>::t)) &&
+           offsetof(KSmem<WIN>, t) == offsetof(KSmem<WIN>, g) + sizeof(KSmem<WIN>::g);
+}
+static_assert(raw_fits<9>() && raw_fits<15>() && raw_fits<21>() && raw_fits<31>(), "two wider windows over g[1] and t");
+
+// Where a level's staged template is: its image window, rows `stride` bytes
+// apart, staged from column sx, of a level w wide; its gradient window
+// likewise (gx0: the window's leftmost column in those terms).
+struct TWin {
+    const uint8_t *st;
+    const uint32_t *sg;
+    int x0, w, sx;
+    int gx0, gw, gsx;
+};
+template <int WIN, int GT>
+__device__ __forceinline__ constexpr int twin_stride() {
+    return GT == VT_GRAD_NONE ? KSmem<WIN>::RS : KSmem<WIN>::JS;
+}
 
 // Shared scratch of a CTA: its warps' windows, and zeros that a lane's run
 // outside the window reads instead of the staged windows (its template
@@ -193,7 +220,7 @@ struct KSmem {
 template <int WIN>
 struct KCta {
     static constexpr int RLZ = WIN / (WIN == 31 ? 1 : 3);
-    uint8_t zj[RLZ * KSmem<WIN>::JS + 16];
+    uint8_t zj[RLZ * KSmem<WIN>::RS + 16];
     uint32_t zg[RLZ * KSmem<WIN>::GS + 4];
     KSmem<WIN> warp[1];  // one per warp of the CTA
 
@@ -244,70 +271,6 @@ __device__ __forceinline__ void run_of(int lane, int i, int &c, int &r0, bool &v
     r0 = band * RL;
 }
 
-// Gradient window of a level without stored gradients (VT_GRAD_NONE): lane c
-// (c <= win) computes the raw Scharr responses of staged column c -- the
-// integers the pyramid kernels would have stored for the replicate-clamped
-// pixel (reflect-101 neighbours) -- and stores them as int16 pairs in the
-// staged gradient window, with the pixel itself in the staged image window
-// (column c of the window at staged column c), so the template is then sampled exactly as from stored int16 gradients.
-//
-// Per image row y the lane forms d(y) = I(y, x+1) - I(y, x-1) and
-// s(y) = 3 I(y, x-1) + 10 I(y, x) + 3 I(y, x+1); the gradient of row y is
-// dx = 3 d(y-1) + 10 d(y) + 3 d(y+1), dy = s(y+1) - s(y-1).  The clamped rows
-// R(k) = clamp(y0 + k) are read once each (a rolling window): for an
-// interior row R(r) its neighbours are R(r-1) and R(r+1); a row at the
-// image's first or last line takes its reflected neighbour (row 1 or h-2)
-// on both sides instead.
-template <int WIN>
-__device__ __forceinline__ void stage_window_otf(const Level &L, int x0, int y0, int lane, uint8_t *st, uint32_t *sg) {
-    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS;
-    const bool ld = lane <= WIN;
-    const int q = clampi(x0 + lane, 0, L.w - 1);
-    const int qm = refl101(q - 1, L.w), qp = refl101(q + 1, L.w);
-    const int hm1 = L.h - 1;
-    auto terms = [&](int y, int &d, int &sm_, int &c) {
-        const uint8_t *rp = L.img + (size_t)y * L.pitch;
-        int a = 0, b = 0, e = 0;
-        if (ld) {
-            a = __ldg(rp + qm);
-            b = __ldg(rp + q);
-            e = __ldg(rp + qp);
-        }
-        d = e - a;
-        sm_ = 3 * (a + e) + 10 * b;
-        c = b;
-    };
-    // reflected neighbours of the first and last image rows (used only when
-    // the window reaches them)
-    int dt = 0, s_t = 0, db = 0, sb = 0, unused;
-    if (y0 <= 0 || hm1 == 0) terms(refl101(-1, L.h), dt, s_t, unused);
-    if (y0 + WIN >= hm1) terms(refl101(L.h, L.h), db, sb, unused);
-    int dm, sm_m, cm, d0, s0, c0;
-    terms(clampi(y0 - 1, 0, hm1), dm, sm_m, cm);
-    terms(clampi(y0, 0, hm1), d0, s0, c0);
-    __syncwarp();
-#pragma unroll
-    for (int r = 0; r <= WIN; ++r) {
-        const int yc = clampi(y0 + r, 0, hm1);
-        int dp, sp, cp;
-        terms(clampi(y0 + r + 1, 0, hm1), dp, sp, cp);
-        const bool top = yc == 0, bot = yc == hm1;
-        const int du = top ? dt : (bot ? db : dm), su = top ? s_t : (bot ? sb : sm_m);
-        const int dd = top ? dt : (bot ? db : dp), sd = top ? s_t : (bot ? sb : sp);
-        const int gx = 3 * (du + dd) + 10 * d0, gy = sd - su;
-        if (ld) {
-            st[r * JS + lane] = (uint8_t)c0;
-            sg[r * GS + lane] = (uint32_t)(uint16_t)(int16_t)gx | ((uint32_t)(uint16_t)(int16_t)gy << 16);
-        }
-        dm = d0;
-        sm_m = s0;
-        d0 = dp;
-        s0 = sp;
-        c0 = cp;
-    }
-    __syncwarp();
-}
-
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
 }
@@ -318,20 +281,20 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Start copying win + 1 rows of NCH 16-byte chunks (row pitch `pitch` bytes,
-// rows y0 .. y0 + win clamped to 0 .. hm1) from `base` to `dst`, the chunks
+// Start copying ROWS rows of NCH 16-byte chunks (row pitch `pitch` bytes,
+// rows from y0 on, clamped to 0 .. hm1) from `base` to `dst`, the chunks
 // below `chunks` of each row.  32 / NCH rows go per step, a lane keeping one
 // chunk of a row: its addresses advance by a constant per step, two
 // instructions per copied chunk (an index split into row and chunk per copy
 // took about 18).
-template <int WIN, int NCH>
+template <int ROWS, int NCH>
 __device__ __forceinline__ void copy_rows(uint32_t dst, const uint8_t *base, int pitch, int y0, int hm1, int chunks,
                                           int lane) {
-    constexpr int RS = 32 / NCH, STEPS = (WIN + RS) / RS;  // rows per step; steps for win + 1 rows
+    constexpr int RS = 32 / NCH, STEPS = (ROWS + RS - 1) / RS;  // rows per step, steps
     const int r = lane / NCH, c = lane - r * NCH;
     const uint32_t d = dst + 16 * lane;
-    const int rows = r < RS && c < chunks ? WIN + 1 - r : 0;  // the lane copies rows r + k RS, k RS < rows
-    if (y0 >= 0 && y0 + WIN <= hm1) {
+    const int rows = r < RS && c < chunks ? ROWS - r : 0;  // the lane copies rows r + k RS, k RS < rows
+    if (y0 >= 0 && y0 + ROWS - 1 <= hm1) {
         const uint8_t *src = base + (size_t)(y0 + r) * pitch + 16 * c;
 #pragma unroll
         for (int k = 0; k < STEPS; ++k) {
@@ -362,14 +325,78 @@ template <int WIN, bool GRAD>
 __device__ __forceinline__ void stage_window(const Level &L, int x0, int y0, int lane, uint8_t *st, uint32_t *sg) {
     const int hm1 = L.h - 1, wx = staged_x(x0, 16);
     __syncwarp();  // every lane is done with what the buffers held
-    copy_rows<WIN, KSmem<WIN>::NC>((uint32_t)__cvta_generic_to_shared(st), L.img + wx, L.pitch, y0, hm1,
+    copy_rows<WIN + 1, KSmem<WIN>::NC>((uint32_t)__cvta_generic_to_shared(st), L.img + wx, L.pitch, y0, hm1,
                                    (L.w - wx + 15) >> 4, lane);
     if constexpr (GRAD) {
         const int gw = staged_x(x0, 4);
-        copy_rows<WIN, KSmem<WIN>::NG>((uint32_t)__cvta_generic_to_shared(sg),
+        copy_rows<WIN + 1, KSmem<WIN>::NG>((uint32_t)__cvta_generic_to_shared(sg),
                                        reinterpret_cast<const uint8_t *>(L.grad + gw), L.gpitch * 4, y0, hm1,
                                        (L.w - gw + 3) >> 2, lane);
     }
+}
+
+// Start staging the image window with top-left (x0, y0) and a border of one
+// pixel on every side (pyramids without gradient planes).
+template <int WIN>
+__device__ __forceinline__ void stage_raw(const Level &L, int x0, int y0, int lane, uint8_t *raw) {
+    const int sx = staged_x(x0 - 1, 16);
+    __syncwarp();
+    copy_rows<WIN + 3, KSmem<WIN>::RS / 16>((uint32_t)__cvta_generic_to_shared(raw), L.img + sx, L.pitch, y0 - 1, L.h - 1,
+                                            (L.w - sx + 15) >> 4, lane);
+}
+
+// Gradient window of a level without stored gradients, from its staged raw
+// window: lane c (c <= win) computes the raw Scharr responses of window
+// column c -- the integers the pyramid kernels would have stored for the
+// replicate-clamped pixel (reflect-101 neighbours, all inside the raw window)
+// -- and stores them as int16 pairs, so the template is then sampled exactly
+// as from stored int16 gradients.
+//
+// Per image row y the lane forms d(y) = I(y, x+1) - I(y, x-1) and
+// s(y) = 3 I(y, x-1) + 10 I(y, x) + 3 I(y, x+1); the gradient of row y is
+// dx = 3 d(y-1) + 10 d(y) + 3 d(y+1), dy = s(y+1) - s(y-1).  Raw row k holds
+// image row clamp(y0 - 1 + k); the rows are read once each (a rolling
+// window): for an interior row its neighbours are the raw rows above and
+// below; a row at the image's first or last line takes its reflected
+// neighbour (row 1 or h-2) on both sides instead.
+template <int WIN>
+__device__ __forceinline__ void gradients_from_raw(const uint8_t *raw, int w, int h, int x0, int y0, int lane,
+                                                   uint32_t *sg) {
+    constexpr int RS = KSmem<WIN>::RS, GS = KSmem<WIN>::GS;
+    if (lane <= WIN) {
+        const int sx = staged_x(x0 - 1, 16), hm1 = h - 1;
+        const int q = clampi(x0 + lane, 0, w - 1);
+        const uint8_t *pm = raw + refl101(q - 1, w) - sx, *p0 = raw + q - sx, *pp = raw + refl101(q + 1, w) - sx;
+        auto terms = [&](int k, int &d, int &s) {  // of raw row k
+            const int a = pm[k * RS], b = p0[k * RS], e = pp[k * RS];
+            d = e - a;
+            s = 3 * (a + e) + 10 * b;
+        };
+        // reflected neighbours of the first and last image rows (used only when
+        // the window reaches them)
+        int dt = 0, st = 0, db = 0, sb = 0;
+        if (y0 <= 0 || hm1 == 0) terms(refl101(-1, h) - y0 + 1, dt, st);
+        if (y0 + WIN >= hm1) terms(refl101(h, h) - y0 + 1, db, sb);
+        int dm, sm, d0, s0;
+        terms(0, dm, sm);
+        terms(1, d0, s0);
+#pragma unroll
+        for (int r = 0; r <= WIN; ++r) {
+            const int yc = clampi(y0 + r, 0, hm1);
+            int dp, sp;
+            terms(r + 2, dp, sp);
+            const bool top = yc == 0, bot = yc == hm1;
+            const int du = top ? dt : (bot ? db : dm), su = top ? st : (bot ? sb : sm);
+            const int dd = top ? dt : (bot ? db : dp), sd = top ? st : (bot ? sb : sp);
+            const int gx = 3 * (du + dd) + 10 * d0, gy = sd - su;
+            sg[r * GS + lane] = (uint32_t)(uint16_t)(int16_t)gx | ((uint32_t)(uint16_t)(int16_t)gy << 16);
+            dm = d0;
+            sm = s0;
+            d0 = dp;
+            s0 = sp;
+        }
+    }
+    __syncwarp();
 }
 
 // Stage the footprint of J with top-left (x0, y0) and wait for it (and for
@@ -398,10 +425,9 @@ __device__ __forceinline__ void run_columns(int x0, int w, int sx, int c, int &o
 // sampled at fractional offset (ax, ay) from the staged windows, zero for
 // samples outside the window.
 template <int WIN, int GT>
-__device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_t *st, const uint32_t *sg, int x0,
-                                                int w, float ax, float ay, int lane, float (&T)[KRuns<WIN>::NS],
-                                                float2 (&G)[KRuns<WIN>::NS]) {
-    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
+__device__ __forceinline__ void sample_template(const KCta<WIN> &C, const TWin &W, float ax, float ay, int lane,
+                                                float (&T)[KRuns<WIN>::NS], float2 (&G)[KRuns<WIN>::NS]) {
+    constexpr int TS = twin_stride<WIN, GT>(), GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     // staged gradient words are int16 pairs when computed in place
     constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
 #pragma unroll
@@ -410,19 +436,19 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const uint8_
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
         int o0, o1;
-        run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
-        const uint8_t *j0 = valid ? st + r0 * JS + o0 : C.zj, *j1 = valid ? st + r0 * JS + o1 : C.zj;
-        const int dg = staged_x(x0, 16) - staged_x(x0, 4);
-        const uint32_t *g0 = valid ? sg + r0 * GS + o0 + dg : C.zg, *g1 = valid ? sg + r0 * GS + o1 + dg : C.zg;
+        run_columns<WIN>(W.x0, W.w, W.sx, c, o0, o1);
+        const uint8_t *j0 = valid ? W.st + r0 * TS + o0 : C.zj, *j1 = valid ? W.st + r0 * TS + o1 : C.zj;
+        run_columns<WIN>(W.gx0, W.gw, W.gsx, c, o0, o1);
+        const uint32_t *g0 = valid ? W.sg + r0 * GS + o0 : C.zg, *g1 = valid ? W.sg + r0 * GS + o1 : C.zg;
         float pi = 0.f;
         float2 pg = pair(0.f);
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = px(j0[r * JS]);
+            const float mv = px(j0[r * TS]);
             float2 gl, gr;
             unpack_grad<GTS>(g0[r * GS], gl.x, gl.y);
             unpack_grad<GTS>(g1[r * GS], gr.x, gr.y);
-            const float hi = fmaf(ax, px_minus(j1[r * JS], mv), mv);
+            const float hi = fmaf(ax, px_minus(j1[r * TS], mv), mv);
             const float2 hg = __ffma2_rn(pair(ax), sub2(gr, gl), gl);
             if (r > 0) {
                 T[i * RL + r - 1] = fmaf(ay, hi - pi, pi);  // zero for a run outside the window
@@ -538,30 +564,42 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// The lane's samples of one staged template row pair in FP64: horizontal
-// lerps of row r of the template image and gradient windows (d: the right
-// neighbour's distance, 0 where it is clamped).
+// The lane's run c, r0 of a staged template in FP64: horizontal lerps of its
+// row r of the image and gradient windows.
 template <int WIN, int GT>
-__device__ __forceinline__ void tmpl_row64(const uint8_t *tr, const uint32_t *gr, int d, int r, double ax, double unit,
-                                           double &hT, double &hGX, double &hGY) {
-    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS;
-    constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
-    const double t0 = (double)tr[r * JS], t1 = (double)tr[r * JS + d];
-    float gx0, gy0, gx1, gy1;
-    unpack_grad<GTS>(gr[r * GS], gx0, gy0);
-    unpack_grad<GTS>(gr[r * GS + d], gx1, gy1);
-    const double x0 = (double)gx0 * unit, x1 = (double)gx1 * unit, y0 = (double)gy0 * unit, y1 = (double)gy1 * unit;
-    hT = fma(ax, t1 - t0, t0);
-    hGX = fma(ax, x1 - x0, x0);
-    hGY = fma(ax, y1 - y0, y0);
-}
+struct Run64 {
+    const uint8_t *t0, *t1;
+    const uint32_t *g0, *g1;
+
+    __device__ __forceinline__ Run64(const TWin &W, int c, int r0) {
+        int o0, o1;
+        run_columns<WIN>(W.x0, W.w, W.sx, c, o0, o1);
+        t0 = W.st + r0 * twin_stride<WIN, GT>() + o0;
+        t1 = W.st + r0 * twin_stride<WIN, GT>() + o1;
+        run_columns<WIN>(W.gx0, W.gw, W.gsx, c, o0, o1);
+        g0 = W.sg + r0 * KSmem<WIN>::GS + o0;
+        g1 = W.sg + r0 * KSmem<WIN>::GS + o1;
+    }
+    __device__ __forceinline__ void row(int r, double ax, double unit, double &hT, double &hGX, double &hGY) const {
+        constexpr int TS = twin_stride<WIN, GT>(), GS = KSmem<WIN>::GS;
+        constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
+        const double a = (double)t0[r * TS], b = (double)t1[r * TS];
+        float gx0, gy0, gx1, gy1;
+        unpack_grad<GTS>(g0[r * GS], gx0, gy0);
+        unpack_grad<GTS>(g1[r * GS], gx1, gy1);
+        const double x0 = (double)gx0 * unit, x1 = (double)gx1 * unit, y0 = (double)gy0 * unit, y1 = (double)gy1 * unit;
+        hT = fma(ax, b - a, a);
+        hGX = fma(ax, x1 - x0, x0);
+        hGY = fma(ax, y1 - y0, y0);
+    }
+};
 
 // G of the level's template in FP64 (grey levels per pixel), every lane
 // holding the totals.
 template <int WIN, int GT>
-__device__ __forceinline__ void template_G64(double ax, double ay, int tx0, int tw, int lane, const uint8_t *st,
-                                             const uint32_t *sg, double &g11, double &g12, double &g22) {
-    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
+__device__ __forceinline__ void template_G64(double ax, double ay, const TWin &W, int lane, double &g11, double &g12,
+                                             double &g22) {
+    constexpr int RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     constexpr double unit = (double)grad_unit<GT>();
     double a11 = 0.0, a12 = 0.0, a22 = 0.0;
 #pragma unroll 1
@@ -570,16 +608,13 @@ __device__ __forceinline__ void template_G64(double ax, double ay, int tx0, int 
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
         if (!valid) continue;
-        int t0, t1;
-        run_columns<WIN>(tx0, tw, staged_x(tx0, 16), c, t0, t1);
-        const uint8_t *tr = st + r0 * JS + t0;
-        const uint32_t *gr = sg + r0 * GS + t0 + staged_x(tx0, 16) - staged_x(tx0, 4);
+        const Run64<WIN, GT> run(W, c, r0);
         double pT, pX, pY;
-        tmpl_row64<WIN, GT>(tr, gr, t1 - t0, 0, ax, unit, pT, pX, pY);
+        run.row(0, ax, unit, pT, pX, pY);
 #pragma unroll 1
         for (int r = 1; r <= RL; ++r) {
             double hT, hX, hY;
-            tmpl_row64<WIN, GT>(tr, gr, t1 - t0, r, ax, unit, hT, hX, hY);
+            run.row(r, ax, unit, hT, hX, hY);
             const double gx = fma(ay, hX - pX, pX), gy = fma(ay, hY - pY, pY);
             a11 = fma(gx, gx, a11);
             a12 = fma(gx, gy, a12);
@@ -597,10 +632,9 @@ __device__ __forceinline__ void template_G64(double ax, double ay, int tx0, int 
 // The eight footprint moments of cell_moments in FP64, the template sampled
 // in FP64 from its staged windows (grey levels per pixel).
 template <int WIN, int GT>
-__device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, double ax, double ay, int tx0,
-                                               int tw, int lane, const uint8_t *st, const uint32_t *sg,
-                                               KSmem<WIN> &sm, double (&m)[8]) {
-    constexpr int JS = KSmem<WIN>::JS, GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
+__device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, double ax, double ay, const TWin &W,
+                                               int lane, KSmem<WIN> &sm, double (&m)[8]) {
+    constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     constexpr double unit = (double)grad_unit<GT>();
     stage_footprint<WIN>(L, x0, y0, lane, sm);
     double a[8];
@@ -612,21 +646,18 @@ __device__ __forceinline__ void cell_moments64(const Level &L, int x0, int y0, d
         bool valid;
         run_of<WIN>(lane, i, c, r0, valid);
         if (!valid) continue;
-        int t0, t1;
-        run_columns<WIN>(tx0, tw, staged_x(tx0, 16), c, t0, t1);
-        const uint8_t *tr = st + r0 * JS + t0;
-        const uint32_t *gr = sg + r0 * GS + t0 + staged_x(tx0, 16) - staged_x(tx0, 4);
+        const Run64<WIN, GT> run(W, c, r0);
         int o0, o1;
         run_columns<WIN>(x0, L.w, staged_x(x0, 16), c, o0, o1);
         const uint8_t *j0 = &sm.j[r0 * JS + o0], *j1 = &sm.j[r0 * JS + o1];
         double pT, pX, pY;
-        tmpl_row64<WIN, GT>(tr, gr, t1 - t0, 0, ax, unit, pT, pX, pY);
+        run.row(0, ax, unit, pT, pX, pY);
         double pmv = (double)j0[0];
         double pdx = (double)j1[0] - pmv;
 #pragma unroll 1
         for (int r = 1; r <= RL; ++r) {
             double hT, hX, hY;
-            tmpl_row64<WIN, GT>(tr, gr, t1 - t0, r, ax, unit, hT, hX, hY);
+            run.row(r, ax, unit, hT, hX, hY);
             const double T = fma(ay, hT - pT, pT), gx = fma(ay, hX - pX, pX), gy = fma(ay, hY - pY, pY);
             const double mv = (double)j0[r * JS];
             const double dx = (double)j1[r * JS] - mv;
@@ -662,9 +693,8 @@ struct Level64 {
 // iterations from the level's guess (gx, gy).
 template <int WIN, int GT>
 __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_iters, const float eps2,
-                                              const float min_eig, float ux, float uy, float gx, float gy, int tx0,
-                                              int tw, int lane, const uint8_t *st, const uint32_t *sg,
-                                              KSmem<WIN> *smp) {
+                                              const float min_eig, float ux, float uy, float gx, float gy,
+                                              const TWin &W, int lane, KSmem<WIN> *smp) {
     constexpr int HW = WIN / 2;
     constexpr double N = (double)(WIN * WIN);
     KSmem<WIN> &sm = *smp;
@@ -675,7 +705,7 @@ __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_i
     o.nx = o.ny = 0.0;
     const double ax = (double)(ux - floorf(ux)), ay = (double)(uy - floorf(uy));
     double G11, G12, G22;
-    template_G64<WIN, GT>(ax, ay, tx0, tw, lane, st, sg, G11, G12, G22);
+    template_G64<WIN, GT>(ax, ay, W, lane, G11, G12, G22);
     const double det64 = G11 * G22 - G12 * G12;
     const double lmax64 = 0.5 * (G11 + G22 + sqrt((G11 - G22) * (G11 - G22) + 4.0 * G12 * G12));
     const double lmin64 = det64 / lmax64 / (N * 65025.0);
@@ -698,7 +728,7 @@ __device__ __forceinline__ Level64 track_level64(const Level Jl, const int max_i
         const double fx = floor(qx), fy = floor(qy);
         const int ix = (int)fx - HW, iy = (int)fy - HW;
         if (ix != cx || iy != cy) {
-            cell_moments64<WIN, GT>(Jl, ix, iy, ax, ay, tx0, tw, lane, st, sg, sm, m);
+            cell_moments64<WIN, GT>(Jl, ix, iy, ax, ay, W, lane, sm, m);
             cx = ix;
             cy = iy;
             ++o.sweeps;
@@ -779,8 +809,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
     // template.  Two commit groups per level, so the waits below count them.
     for (int l = L; l >= 0; --l) {
         const float ax = ux - ufx, ay = uy - ufy;
-        int tx0 = (int)ufx - HW;  // leftmost template column
-        const int ty0 = (int)ufy - HW, w_I = tw;
+        const int tx0 = (int)ufx - HW, ty0 = (int)ufy - HW, w_I = tw;  // the template's window
         const float qx0 = ux + gx, qy0 = uy + gy;  // the level's first footprint position
         float limx = 0.f, limy = 0.f;              // footprint positions lie in [-HW, limx] x [-HW, limy]
         bool inside = false;
@@ -804,23 +833,30 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             ux = ux0 * s, uy = uy0 * s;
             ufx = floorf(ux), ufy = floorf(uy);
             tw = In.w;
-            if constexpr (GT != VT_GRAD_NONE)
+            if constexpr (GT == VT_GRAD_NONE)
+                stage_raw<WIN>(In, (int)ufx - HW, (int)ufy - HW, lane, sm.raw((l - 1) & 1));
+            else
                 stage_window<WIN, true>(In, (int)ufx - HW, (int)ufy - HW, lane, sm.t[(l - 1) & 1], sm.g[(l - 1) & 1]);
         }
         cp_async_commit();
         if (l == L) continue;
-        uint8_t *st = sm.t[l & 1];
-        uint32_t *sg = sm.g[l & 1];
+        TWin W;
+        W.x0 = tx0, W.w = w_I;
+        cp_async_wait<2>();
+        __syncwarp();
         if constexpr (GT == VT_GRAD_NONE) {
-            __syncwarp();
-            stage_window_otf<WIN>(I[l], tx0, ty0, lane, st, sg);
-            tx0 = 0;  // staged column by column from 0, clamped already
-            sample_template<WIN, GT>(C, st, sg, 0, WIN + 1, ax, ay, lane, T, G);
+            gradients_from_raw<WIN>(sm.raw(l & 1), w_I, I[l].h, tx0, ty0, lane, sm.g[0]);
+            W.st = sm.raw(l & 1) + KSmem<WIN>::RS;
+            W.sg = sm.g[0];
+            W.sx = staged_x(tx0 - 1, 16);
+            W.gx0 = 0, W.gw = WIN + 1, W.gsx = 0;  // window columns, clamped already
         } else {
-            cp_async_wait<2>();
-            __syncwarp();
-            sample_template<WIN, GT>(C, st, sg, tx0, w_I, ax, ay, lane, T, G);
+            W.st = sm.t[l & 1];
+            W.sg = sm.g[l & 1];
+            W.sx = staged_x(tx0, 16);
+            W.gx0 = tx0, W.gw = w_I, W.gsx = staged_x(tx0, 4);
         }
+        sample_template<WIN, GT>(C, W, ax, ay, lane, T, G);
         ++o.tmpl;
         float2 aii = pair(0.f);
         float a12 = 0.f;
@@ -849,8 +885,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             } else {
                 cp_async_wait<0>();  // the first footprint started above: sm.j is staged anew
                 const Level64 r = track_level64<WIN, GT>(Jl, P.max_iters, P.eps2, P.min_eig, ux0 * pow2neg(l),
-                                                         uy0 * pow2neg(l), gx, gy, tx0,
-                                                         GT == VT_GRAD_NONE ? WIN + 1 : w_I, lane, st, sg, &sm);
+                                                         uy0 * pow2neg(l), gx, gy, W, lane, &sm);
                 cfx = kNone;
                 o.lmin = r.lmin;
                 o.iters += r.iters;
@@ -978,7 +1013,13 @@ template <int WIN, int GT, bool F64>
 __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, const KParams &P, float ux0,
                                                 float uy0, bool fb, bool has_guess, float gux, float guy, int lane,
                                                 const KCta<WIN> &C, KSmem<WIN> &sm, KOut &o) {
-    const Level *A = I, *B = J;
+    // the two level tables next to the warp: a level's fields are one shared
+    // load away, not a chain of global ones
+    static_assert(sizeof(Level) * VT_MAX_LEVELS == 16 * 16, "16 lanes copy a table");
+    __syncwarp();
+    reinterpret_cast<uint4 *>(sm.lv)[lane] = reinterpret_cast<const uint4 *>(lane < 16 ? I : J)[lane & 15];
+    __syncwarp();
+    const Level *A = sm.lv[0], *B = sm.lv[1];
     float x = ux0, y = uy0;
     const int npass = fb ? 2 : 1;
 #pragma unroll 1
@@ -991,8 +1032,8 @@ __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, 
             if (!r.status) return;
             x = r.x;
             y = r.y;
-            A = J;
-            B = I;
+            A = sm.lv[1];
+            B = sm.lv[0];
         } else {
             o.iters += r.iters;
             o.tmpl += r.tmpl;
