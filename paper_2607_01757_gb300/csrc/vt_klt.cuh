@@ -183,6 +183,11 @@ struct KSmem {
     static constexpr int GS = NG * 4;                         // staged gradient row stride in words
     static_assert(GS >= 3 + WIN + 1, "a staged gradient row covers the window row");
     Level lv[2][VT_MAX_LEVELS];  // the point's two pyramids
+    // moments of the level's footprint cells that the position left, by the
+    // parity of the cell: neighbouring cells never share an entry, so a point
+    // that hovers at a cell's edge or corner comes back to kept moments
+    float2 cell_m[4][4];
+    int2 cell_at[4];
     uint8_t j[(WIN + 1) * JS];
     uint32_t g[2][(WIN + 1) * GS];
     uint8_t t[2][(WIN + 1) * JS];
@@ -795,9 +800,10 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         gx = (gux - ux0) * s;
         gy = (guy - uy0) * s;
     }
-    // integer part of the footprint position last staged in sm.j (unknown: NaN)
+    // integer part of the current footprint cell (unknown: NaN)
     constexpr float kNone = __builtin_nanf("");
     float cfx = kNone, cfy = kNone;
+    bool staged = true;  // whether sm.j holds that cell's footprint
     // the template started by the previous iteration: position, its floor, the level's width
     float ux = 0.f, uy = 0.f, ufx = 0.f, ufy = 0.f;
     int tw = 0;
@@ -823,6 +829,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             if (inside) {
                 cfx = floorf(qx0);
                 cfy = floorf(qy0);
+                staged = true;
                 stage_window<WIN, false>(Jl, (int)cfx - HW, (int)cfy - HW, lane, sm.j, nullptr);
             }
             cp_async_commit();
@@ -936,6 +943,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         // step takes the full test (0).
         constexpr unsigned kOne = 0x3f800000u;
         unsigned cell_end = cfx >= limx || cfy >= limy ? 0u : kOne;
+        bool left_cell = false;  // whether sm.cell_* hold this level's entries
         for (int k = 1;; ++k) {
             const float bxy = bx * by;
             float2 b = __ffma2_rn(pair(-bx), m[1], m[0]);
@@ -957,10 +965,29 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
                 }
                 const float fx = floorf(qx), fy = floorf(qy);
                 if (fx != cfx || fy != cfy) {
+                    // every lane stores and reads back the same values
+                    const int ix = (int)fx, iy = (int)fy, px = (int)cfx, py = (int)cfy;
+                    const int slot = (ix & 1) | (iy & 1) << 1, old = (px & 1) | (py & 1) << 1;
+                    if (!left_cell) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) sm.cell_at[q] = make_int2(INT_MIN, INT_MIN);
+                        left_cell = true;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) sm.cell_m[old][q] = m[q];
+                    sm.cell_at[old] = make_int2(px, py);
                     cfx = fx, cfy = fy;
-                    stage_footprint<WIN>(Jl, (int)fx - HW, (int)fy - HW, lane, sm);
-                    cell_moments<WIN>((int)fx - HW, Jl.w, lane, T, G, sm, m);
-                    ++o.sweeps;
+                    const int2 at = sm.cell_at[slot];
+                    if (at.x == ix && at.y == iy) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) m[q] = sm.cell_m[slot][q];
+                        staged = false;
+                    } else {
+                        stage_footprint<WIN>(Jl, ix - HW, iy - HW, lane, sm);
+                        cell_moments<WIN>(ix - HW, Jl.w, lane, T, G, sm, m);
+                        ++o.sweeps;
+                        staged = true;
+                    }
                     bx = qx - fx, by = qy - fy;
                     cell_end = fx >= limx || fy >= limy ? 0u : kOne;
                 }
@@ -997,7 +1024,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             if (want_err) {
                 const float fx = floorf(o.x), fy = floorf(o.y);
                 const int ix = (int)fx - HW, iy = (int)fy - HW;
-                if (fx != cfx || fy != cfy) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
+                if (fx != cfx || fy != cfy || !staged) stage_footprint<WIN>(J[0], ix, iy, lane, sm);
                 o.err = abs_residual<WIN>(C, ix, J[0].w, o.x - fx, o.y - fy, lane, T, sm) * kImgUnscale / N;
                 ++o.errp;
             }
