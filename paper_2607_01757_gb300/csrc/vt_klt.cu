@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(KLT_WARPS * 32, KltOcc<WIN>::min_blocks) k_klt
     KSmem<WIN> &sm = C.warp[threadIdx.x >> 5];
     const int pt = blockIdx.x * KLT_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    pdl_wait();  // the points and pyramids may be the previous kernel's output
     if (pt >= A.n) return;
     if (F64 && A.status[pt] != kStatusPending) return;
     const float2 p = A.pts_in[pt];
@@ -77,7 +78,9 @@ static void launch_pass(const KltArgs &A, cudaStream_t s) {
         }();
         (void)attr;
     }
-    k_klt<WIN, GT, FB, F64><<<blocks, KLT_WARPS * 32, smem, s>>>(A);
+    // launched while the stream's previous kernel ends (programmatic dependent
+    // launch): the tables are filled meanwhile
+    launch_pdl(k_klt<WIN, GT, FB, F64>, blocks, KLT_WARPS * 32, smem, s, true, A);
 }
 
 // The FP32 launch, then (only when an accepted template can be
