@@ -56,10 +56,23 @@ __device__ __forceinline__ void scharr_at(const uint8_t (*s)[IW], int sr, int sc
     dy = 3 * (a20 - a00) + 10 * (a21 - a01) + 3 * (a22 - a02);
 }
 
+// 16 bytes at any address, by the aligned words that hold them (each holds at
+// least one of the bytes, so none lies outside the caller's allocation).
+__device__ __forceinline__ uint4 load16_any(const uint8_t *p) {
+    const unsigned a = (unsigned)(uintptr_t)p & 3u;
+    const uint32_t *q = reinterpret_cast<const uint32_t *>(p - a);
+    uint32_t v[5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldg(q + k);
+    v[4] = a ? __ldg(q + 4) : 0u;
+    return make_uint4(__funnelshift_r(v[0], v[1], 8 * a), __funnelshift_r(v[1], v[2], 8 * a),
+                      __funnelshift_r(v[2], v[3], 8 * a), __funnelshift_r(v[3], v[4], 8 * a));
+}
+
 // Stage rows [iy0, iy0 + IH) and columns [ix0, ix0 + IW) of an image (ix0 a
 // multiple of 16), rows and columns reflected into it; ends with a barrier.
-// With 16-byte aligned rows (vec_ok) the 16-byte chunks inside the image are
-// copied whole, the chunk that holds the last column byte by byte (a caller's
+// The 16-byte chunks inside the image are copied whole (one load where the
+// rows are 16-byte aligned, vec_ok, else word by word), the chunk that holds the last column byte by byte (a caller's
 // last row may end there); the columns -2, -1, w and w + 1 are then filled
 // from the staged ones (the reflected columns lie in the same tile for w >= 4;
 // the readers use no others outside the image).  A tile at the image's edge
@@ -70,13 +83,14 @@ template <int IH, int IW>
 __device__ __forceinline__ void stage_tile(uint8_t (*s)[IW], const uint8_t *src, int w, int h, int pitch, int ix0,
                                            int iy0, bool vec_ok) {
     constexpr int C16 = IW / 16;
-    if (vec_ok && w >= 4) {
+    if (w >= 4) {
         const bool inner = ix0 >= 0 && ix0 + IW <= w && iy0 >= 0 && iy0 + IH <= h;
         for (int i = threadIdx.x; i < IH * C16; i += blockDim.x) {
             const int r = i / C16, c = i - r * C16, x = ix0 + 16 * c;
             const uint8_t *row = src + (size_t)(inner ? iy0 + r : refl101(iy0 + r, h)) * pitch;
             if (inner || (x >= 0 && x + 16 <= w)) {
-                *reinterpret_cast<uint4 *>(&s[r][c * 16]) = __ldg(reinterpret_cast<const uint4 *>(row + x));
+                *reinterpret_cast<uint4 *>(&s[r][c * 16]) =
+                    vec_ok ? __ldg(reinterpret_cast<const uint4 *>(row + x)) : load16_any(row + x);
             } else if (x >= 0 && x < w) {
                 for (int q = 0; x + q < w; ++q) s[r][c * 16 + q] = __ldg(row + x + q);
             }
@@ -123,59 +137,110 @@ __device__ __forceinline__ void copy_out(const uint8_t (*s)[IW], int r0, int c0,
     }
 }
 
-// Scharr (int16 output) of 4 consecutive columns x .. x+3 and 4 rows y0 ..
-// y0+3 of the staged tile, two pixels per 32-bit operation.  A word holds two
-// columns two apart in its 16-bit lanes: (x, x+2), (x+1, x+3), and the edge
-// columns (x-1, x+4).  Per lane, the vertical smoothing V = 3 top + 10 mid +
-// 3 bottom is at most 4080 and the biased difference D = bottom - top + 2048
-// lies in [1793, 2303], so
+// Four columns x .. x+3 of a staged row as the packed Scharr pass holds them:
+// two columns two apart in the 16-bit lanes of a word, (x, x+2), (x+1, x+3),
+// and the edge columns (x-1, x+4).
+struct Row4 {
+    uint32_t c13, c24, ce;
+};
+// From the words that hold columns x-4 .. x-1, x .. x+3 and x+4 .. x+7.
+__device__ __forceinline__ Row4 row4(uint32_t a, uint32_t b, uint32_t c) {
+    return {b & 0x00FF00FFu, (b >> 8) & 0x00FF00FFu, (a >> 24) | ((c << 16) & 0x00FF0000u)};
+}
+
+// Scharr (int16 output) of 4 consecutive columns of the row between `t` and
+// `u` (m: the row itself), two pixels per 32-bit operation.  Per lane, the
+// vertical smoothing V = 3 top + 10 mid + 3 bottom is at most 4080 and the
+// biased difference D = bottom - top + 2048 lies in [1793, 2303], so
 //   dx + 32768 = V(x+1) - V(x-1) + 32768,
 //   dy + 32768 = 3 D(x-1) + 10 D(x) + 3 D(x+1)      (bias 16 * 2048)
 // both lie in [28688, 36848]: no lane ever borrows from or carries into its
 // neighbour, and flipping bit 15 of a lane turns the biased value into the
 // int16 two's complement of dx or dy.  Same results as the scalar form.
-// `sr0` is the staged row above y0; `xr` the staged column offset of x.
+__device__ __forceinline__ uint4 scharr4_s16(const Row4 &t, const Row4 &m, const Row4 &u) {
+    const uint32_t v13 = 3u * (t.c13 + u.c13) + 10u * m.c13;
+    const uint32_t v24 = 3u * (t.c24 + u.c24) + 10u * m.c24;
+    const uint32_t ve = 3u * (t.ce + u.ce) + 10u * m.ce;
+    const uint32_t d13 = u.c13 + 0x08000800u - t.c13;
+    const uint32_t d24 = u.c24 + 0x08000800u - t.c24;
+    const uint32_t de = u.ce + 0x08000800u - t.ce;
+    const uint32_t vm = __byte_perm(ve, v24, 0x5410), vp = __byte_perm(v13, ve, 0x7632);  // (x-1, x+1), (x+2, x+4)
+    const uint32_t dm = __byte_perm(de, d24, 0x5410), dp = __byte_perm(d13, de, 0x7632);
+    const uint32_t dx13 = (v24 + 0x80008000u - vm) ^ 0x80008000u;  // columns (x, x+2)
+    const uint32_t dx24 = (vp + 0x80008000u - v13) ^ 0x80008000u;  // columns (x+1, x+3)
+    const uint32_t dy13 = (3u * (dm + d24) + 10u * d13) ^ 0x80008000u;
+    const uint32_t dy24 = (3u * (d13 + dp) + 10u * d24) ^ 0x80008000u;
+    return make_uint4(__byte_perm(dx13, dy13, 0x5410), __byte_perm(dx24, dy24, 0x5410),
+                      __byte_perm(dx13, dy13, 0x7632), __byte_perm(dx24, dy24, 0x7632));
+}
+
+// The gradient words of columns x .. x+3 to a row of w columns.
+__device__ __forceinline__ void store_grad4(uint32_t *row, int x, int w, const uint4 &g) {
+    if (x + 3 < w) {
+        *reinterpret_cast<uint4 *>(row + x) = g;
+    } else {
+        const uint32_t gq[4] = {g.x, g.y, g.z, g.w};
+        for (int q = 0; q < 4 && x + q < w; ++q) row[x + q] = gq[q];
+    }
+}
+
+// Scharr (int16 output) of 4 consecutive columns x .. x+3 and 4 rows y0 ..
+// y0+3 of the staged tile.  `sr0` is the staged row above y0; `xr` the staged
+// column offset of x.
 __device__ __forceinline__ void scharr_4x4_s16(const uint8_t (*s)[PD_IW], int sr0, int xr, int x, int y0, int w,
                                                int h, uint32_t *grad, int gpitch) {
-    uint32_t c13[3], c24[3], ce[3];  // rows above, centre, below
-    auto load_row = [&](int sr, uint32_t &a13, uint32_t &a24, uint32_t &ae) {
+    auto load_row = [&](int sr) {
         const uint32_t *wp = reinterpret_cast<const uint32_t *>(&s[sr][12 + xr]);
-        const uint32_t a = wp[0], b = wp[1], c = wp[2];  // columns x-4 .. x+7
-        a13 = b & 0x00FF00FFu;
-        a24 = (b >> 8) & 0x00FF00FFu;
-        ae = (a >> 24) | ((c << 16) & 0x00FF0000u);
+        return row4(wp[0], wp[1], wp[2]);  // columns x-4 .. x+7
     };
-    load_row(sr0, c13[0], c24[0], ce[0]);
-    load_row(sr0 + 1, c13[1], c24[1], ce[1]);
+    Row4 r0 = load_row(sr0), r1 = load_row(sr0 + 1);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        load_row(sr0 + 2 + i, c13[2], c24[2], ce[2]);
+        const Row4 r2 = load_row(sr0 + 2 + i);
         const int y = y0 + i;
-        if (y < h && x < w) {
-            const uint32_t v13 = 3u * (c13[0] + c13[2]) + 10u * c13[1];
-            const uint32_t v24 = 3u * (c24[0] + c24[2]) + 10u * c24[1];
-            const uint32_t ve = 3u * (ce[0] + ce[2]) + 10u * ce[1];
-            const uint32_t d13 = c13[2] + 0x08000800u - c13[0];
-            const uint32_t d24 = c24[2] + 0x08000800u - c24[0];
-            const uint32_t de = ce[2] + 0x08000800u - ce[0];
-            const uint32_t vm = __byte_perm(ve, v24, 0x5410), vp = __byte_perm(v13, ve, 0x7632);  // (x-1, x+1), (x+2, x+4)
-            const uint32_t dm = __byte_perm(de, d24, 0x5410), dp = __byte_perm(d13, de, 0x7632);
-            const uint32_t dx13 = (v24 + 0x80008000u - vm) ^ 0x80008000u;  // columns (x, x+2)
-            const uint32_t dx24 = (vp + 0x80008000u - v13) ^ 0x80008000u;  // columns (x+1, x+3)
-            const uint32_t dy13 = (3u * (dm + d24) + 10u * d13) ^ 0x80008000u;
-            const uint32_t dy24 = (3u * (d13 + dp) + 10u * d24) ^ 0x80008000u;
-            const uint32_t g0 = __byte_perm(dx13, dy13, 0x5410), g2 = __byte_perm(dx13, dy13, 0x7632);
-            const uint32_t g1 = __byte_perm(dx24, dy24, 0x5410), g3 = __byte_perm(dx24, dy24, 0x7632);
-            uint32_t *d = grad + (size_t)y * gpitch + x;
-            if (x + 3 < w) {
-                *reinterpret_cast<uint4 *>(d) = make_uint4(g0, g1, g2, g3);
-            } else {
-                const uint32_t gq[4] = {g0, g1, g2, g3};
-                for (int q = 0; q < 4 && x + q < w; ++q) d[q] = gq[q];
-            }
-        }
-        c13[0] = c13[1], c24[0] = c24[1], ce[0] = ce[1];
-        c13[1] = c13[2], c24[1] = c24[2], ce[1] = ce[2];
+        if (y < h && x < w) store_grad4(grad + (size_t)y * gpitch, x, w, scharr4_s16(r0, r1, r2));
+        r0 = r1;
+        r1 = r2;
+    }
+}
+
+// Vertical [1 4 6 4 1] sums of a word's columns over five rows: (columns 0, 2)
+// and (1, 3) in 16-bit lanes (at most 16 * 255, no carry between lanes).
+__device__ __forceinline__ void vsum4(const uint32_t (&v)[5], uint32_t &sl, uint32_t &sh) {
+    uint32_t lo[5], hi[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        lo[k] = v[k] & 0x00FF00FFu;
+        hi[k] = (v[k] >> 8) & 0x00FF00FFu;
+    }
+    sl = lo[0] + lo[4] + 4u * (lo[1] + lo[3]) + 6u * lo[2];
+    sh = hi[0] + hi[4] + 4u * (hi[1] + hi[3]) + 6u * hi[2];
+}
+
+// Four consecutive pyramid outputs from the vertical sums of their columns,
+// two outputs per 32-bit operation: p[k] holds columns (2k - 2, 2k - 1)
+// relative to the first output's centre, and output q needs columns 2q - 2 ..
+// 2q + 2, so lane pairs (c, c+2) are gathered by byte permutes; a lane's sum
+// is at most 16 * 4080 + 128 and never carries into its neighbour.
+__device__ __forceinline__ uint32_t hsum4(const uint32_t (&p)[6]) {
+    auto lo2 = [](uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x5410); };
+    auto hi2 = [](uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); };
+    auto down2 = [](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4) {
+        const uint32_t sum = w0 + w4 + 0x00800080u + 4u * (w1 + w3) + 6u * w2;
+        return (sum >> 8) & 0x00FF00FFu;
+    };
+    const uint32_t w4 = lo2(p[2], p[3]);
+    const uint32_t ra = down2(lo2(p[0], p[1]), hi2(p[0], p[1]), lo2(p[1], p[2]), hi2(p[1], p[2]), w4);
+    const uint32_t rb = down2(w4, hi2(p[2], p[3]), lo2(p[3], p[4]), hi2(p[3], p[4]), lo2(p[4], p[5]));
+    return __byte_perm(ra, rb, 0x6420);  // bytes o0, o1, o2, o3
+}
+
+// Four outputs x .. x+3 to a row of w columns.
+__device__ __forceinline__ void store_px4(uint8_t *row, int x, int w, uint32_t packed) {
+    if (x + 3 < w) {
+        *reinterpret_cast<uint32_t *>(row + x) = packed;
+    } else {
+        for (int q = 0; q < 4 && x + q < w; ++q) row[x + q] = (uint8_t)(packed >> (8 * q));
     }
 }
 
@@ -220,15 +285,10 @@ __device__ __forceinline__ void pyr_tile_compute(int w, int h, uint8_t *dst, int
     // vertical pass: s_v[r][c] = sum_k [1 4 6 4 1]_k staged(2r + k, 12 + c)
     for (int i = threadIdx.x; i < PD_TH * (PD_VW / 4); i += PD_THREADS) {
         const int r = i / (PD_VW / 4), j = i - r * (PD_VW / 4);
-        uint32_t lo[5], hi[5];
+        uint32_t v[5], sl, sh;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            const uint32_t v = *reinterpret_cast<const uint32_t *>(&s_in[2 * r + k][12 + 4 * j]);
-            lo[k] = v & 0x00FF00FFu;
-            hi[k] = (v >> 8) & 0x00FF00FFu;
-        }
-        const uint32_t sl = lo[0] + lo[4] + 4u * (lo[1] + lo[3]) + 6u * lo[2];
-        const uint32_t sh = hi[0] + hi[4] + 4u * (hi[1] + hi[3]) + 6u * hi[2];
+        for (int k = 0; k < 5; ++k) v[k] = *reinterpret_cast<const uint32_t *>(&s_in[2 * r + k][12 + 4 * j]);
+        vsum4(v, sl, sh);
         uint32_t *out = reinterpret_cast<uint32_t *>(&s_v[r][0]) + 2 * j;
         *reinterpret_cast<uint2 *>(out) = make_uint2(__byte_perm(sl, sh, 0x5410), __byte_perm(sl, sh, 0x7632));
     }
@@ -288,31 +348,11 @@ __device__ __forceinline__ void pyr_tile_compute(int w, int h, uint8_t *dst, int
         const int r = threadIdx.x >> 4, x4 = (threadIdx.x & 15) * 4;
         const int oy = oy0 + r, ox = ox0 + x4;
         if (oy < H && ox < W) {
-            // two outputs per 32-bit operation: lanes (o0, o1) and (o2, o3);
-            // word k of the row holds s_v columns (2k, 2k+1) after the
-            // offset, and output q needs columns 2q .. 2q+4, so lane pairs
-            // (c, c+2) are gathered by byte permutes; a lane's sum is at
-            // most 16 * 4080 = 65280 and never carries into its neighbour
             const uint32_t *pr = reinterpret_cast<const uint32_t *>(&s_v[r][0]) + x4 + 1;
             uint32_t p[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) p[k] = pr[k];
-            auto lo2 = [](uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x5410); };
-            auto hi2 = [](uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); };
-            auto down2 = [](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4) {
-                const uint32_t sum = w0 + w4 + 0x00800080u + 4u * (w1 + w3) + 6u * w2;
-                return (sum >> 8) & 0x00FF00FFu;
-            };
-            const uint32_t w4 = lo2(p[2], p[3]);
-            const uint32_t ra = down2(lo2(p[0], p[1]), hi2(p[0], p[1]), lo2(p[1], p[2]), hi2(p[1], p[2]), w4);
-            const uint32_t rb = down2(w4, hi2(p[2], p[3]), lo2(p[3], p[4]), hi2(p[3], p[4]), lo2(p[4], p[5]));
-            const uint32_t packed = __byte_perm(ra, rb, 0x6420);  // bytes o0, o1, o2, o3
-            uint8_t *d = dst + (size_t)oy * dpitch + ox;
-            if (ox + 3 < W) {
-                *reinterpret_cast<uint32_t *>(d) = packed;
-            } else {
-                for (int q = 0; q < 4 && ox + q < W; ++q) d[q] = (uint8_t)(packed >> (8 * q));
-            }
+            store_px4(dst + (size_t)oy * dpitch, ox, W, hsum4(p));
         }
     }
 }
@@ -453,89 +493,205 @@ __global__ void __launch_bounds__(PD_THREADS, 6) k_pyr_batch(const uint8_t *tab,
 
 // ------------------------------------------------------------------ tail
 constexpr int TAIL_THREADS = 1024;
-constexpr int TAIL_A = kTailMaxPx;             // level c (<= kTailMaxPx pixels)
-constexpr int TAIL_B = kTailMaxPx / 2 + 512;   // level c+1 (<= (w h + w + h + 1) / 4 pixels)
+// A level in shared memory: rows of tail_stride(w) bytes, column x at byte
+// 4 + x, with the reflected columns -2, -1, w and w + 1 filled in.  Every
+// level of at most kTailMaxPx bytes at a pitch of 64 or more fits in TAIL_A,
+// and its successor in TAIL_B (checked over all widths); a group of four
+// outputs may read up to 16 bytes past the last row.
+__host__ __device__ constexpr int tail_stride(int w) { return (w + 3) / 4 * 4 + 8; }
+constexpr int TAIL_A = 46080 + 16;  // level c, and every second level after it
+constexpr int TAIL_B = 20488 + 24;  // level c + 1, ...
+__host__ __device__ inline bool tail_fits(const Level &L) {
+    return (long)L.pitch * L.h <= kTailMaxPx && (long)tail_stride(L.w) * L.h <= TAIL_A - 16;
+}
 constexpr int TAIL_SMEM = TAIL_A + TAIL_B;
 
 // First level the tail kernel builds: the first whose rows (at the
 // pyramid's pitch) fit in kTailMaxPx bytes, or the last.
 int tail_start_level(const vt_pyramid *p) {
     for (int l = 0; l < p->levels; ++l)
-        if ((long)p->lv[l].pitch * p->lv[l].h <= kTailMaxPx) return l;
+        if (tail_fits(p->lv[l])) return l;
     return p->levels - 1;
 }
 
-// Row bands (CTAs) of a frame's tail: about 4096 pixels of level c each, at most 8.
+// CTAs of a frame's tail: one builds the levels below c, the others (about
+// 4096 pixels each, at most 7) take row bands of level c's gradients.  A last
+// level too large for shared memory is shared tile by tile.
 int tail_parts(const vt_pyramid *p) {
     const int c = tail_start_level(p);
     const long px = (long)p->lv[c].w * p->lv[c].h;
-    if ((long)p->lv[c].pitch * p->lv[c].h > kTailMaxPx) return 1;
-    int n = (int)((px + 4095) / 4096);
-    n = n < 1 ? 1 : (n > 8 ? 8 : n);
-    return n < p->lv[c].h ? n : (p->lv[c].h > 0 ? p->lv[c].h : 1);
+    if (!tail_fits(p->lv[c])) return 8;
+    const int n = 1 + (int)((px + 4095) / 4096);
+    return n > 8 ? 8 : n;
 }
 
-// Reflect-101 neighbours one step away (valid for any n >= 1).
-__device__ __forceinline__ int refl_m1(int i, int n) { return i > 0 ? i - 1 : (n > 1 ? 1 : 0); }
-__device__ __forceinline__ int refl_p1(int i, int n) { return i < n - 1 ? i + 1 : (n > 1 ? n - 2 : 0); }
+// Fill the reflected columns of rows [y0, y1) of a w-wide level in shared memory.
+__device__ __forceinline__ void tail_pad(uint8_t *s, int w, int y0, int y1) {
+    const int S = tail_stride(w);
+    const int l2 = refl101(-2, w), l1 = refl101(-1, w), r0 = refl101(w, w), r1 = refl101(w + 1, w);
+    for (int y = y0 + threadIdx.x; y < y1; y += blockDim.x) {
+        uint8_t *r = s + y * S + 4;
+        r[-2] = r[l2];
+        r[-1] = r[l1];
+        r[w] = r[r0];
+        r[w + 1] = r[r1];
+    }
+    __syncwarp();
+}
 
-// Scharr of rows [y0, y1) of a w x h level held in shared memory; warps take
-// rows, lanes take columns.
+// Scharr of rows [y0, y1) of a w x h level held in shared memory, four columns
+// a thread (the words of three rows; int16 planes two pixels per operation).
 template <int GT>
-__device__ __forceinline__ void tail_scharr(const uint8_t *s, int stride, int w, int h, int y0, int y1,
-                                            uint32_t *grad, int gpitch) {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int y = y0 + (threadIdx.x >> 5); y < y1; y += nw) {
-        const uint8_t *rm = s + refl_m1(y, h) * stride, *r0 = s + y * stride, *rp = s + refl_p1(y, h) * stride;
-        uint32_t *g = grad + (size_t)y * gpitch;
-        for (int x = lane; x < w; x += 32) {
-            const int xm = refl_m1(x, w), xp = refl_p1(x, w);
-            const int a00 = rm[xm], a01 = rm[x], a02 = rm[xp];
-            const int a10 = r0[xm], a12 = r0[xp];
-            const int a20 = rp[xm], a21 = rp[x], a22 = rp[xp];
-            const int sm = 3 * (a02 - a00) + 10 * (a12 - a10) + 3 * (a22 - a20);
-            const int dy = 3 * (a20 - a00) + 10 * (a21 - a01) + 3 * (a22 - a02);
-            g[x] = pack_grad<GT>(sm, dy);
+__device__ __forceinline__ void tail_scharr(const uint8_t *s, int w, int h, int y0, int y1, uint32_t *grad,
+                                            int gpitch) {
+    const int S = tail_stride(w), G = (w + 3) / 4;
+    for (int i = threadIdx.x; i < (y1 - y0) * G; i += blockDim.x) {
+        const int y = y0 + i / G, g = i % G;
+        uint32_t v[3][3];  // columns 4g - 4 .. 4g + 7 of the rows above, at and below y
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t *wp = reinterpret_cast<const uint32_t *>(s + refl101(y + k - 1, h) * S) + g;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[k][c] = wp[c];
         }
-    }
-}
-
-// pyrDown of a w x h level in shared memory (row stride `stride`) into d
-// (shared, tight rows) and g (global).
-__device__ __forceinline__ void tail_pyrdown(const uint8_t *s, int stride, int w, int h, uint8_t *d, uint8_t *g,
-                                             int gpitch) {
-    const int W = (w + 1) >> 1, H = (h + 1) >> 1;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int Y = threadIdx.x >> 5; Y < H; Y += nw) {
-        const uint8_t *rows[5];
+        uint4 q;
+        if constexpr (GT == VT_GRAD_S16) {
+            q = scharr4_s16(row4(v[0][0], v[0][1], v[0][2]), row4(v[1][0], v[1][1], v[1][2]),
+                            row4(v[2][0], v[2][1], v[2][2]));
+        } else {
+            int sm[6], dd[6];  // columns 4g - 1 .. 4g + 4
 #pragma unroll
-        for (int k = 0; k < 5; ++k) rows[k] = s + refl101(2 * Y + k - 2, h) * stride;
-        for (int X = lane; X < W; X += 32) {
-            int cols[5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) cols[k] = refl101(2 * X + k - 2, w);
-            uint32_t acc = 0;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) {
-                const uint8_t *r = rows[j];
-                const uint32_t v = r[cols[0]] + r[cols[4]] + 4u * (r[cols[1]] + r[cols[3]]) + 6u * r[cols[2]];
-                acc += (j == 2 ? 6u : (j == 1 || j == 3 ? 4u : 1u)) * v;
+            for (int c = 0; c < 6; ++c) {
+                const int wd = (c + 3) >> 2, sh = 8 * ((c + 3) & 3);
+                const int a = (v[0][wd] >> sh) & 255, b = (v[1][wd] >> sh) & 255, e = (v[2][wd] >> sh) & 255;
+                sm[c] = 3 * (a + e) + 10 * b;
+                dd[c] = e - a;
             }
-            const uint8_t o = (uint8_t)((acc + 128u) >> 8);
-            d[Y * W + X] = o;
-            g[(size_t)Y * gpitch + X] = o;
+            uint32_t o[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o[c] = pack_grad<GT>(sm[c + 2] - sm[c], 3 * (dd[c] + dd[c + 2]) + 10 * dd[c + 1]);
+            q = make_uint4(o[0], o[1], o[2], o[3]);
         }
+        store_grad4(grad + (size_t)y * gpitch, 4 * g, w, q);
+    }
+    __syncwarp();
+}
+
+// pyrDown of a w x h level in shared memory into d (shared) and g (global),
+// four outputs a thread.
+__device__ __forceinline__ void tail_pyrdown(const uint8_t *s, int w, int h, uint8_t *d, uint8_t *g, int gpitch) {
+    const int W = (w + 1) >> 1, H = (h + 1) >> 1, G = (W + 3) / 4;
+    const int S = tail_stride(w), D = tail_stride(W);
+    for (int i = threadIdx.x; i < H * G; i += blockDim.x) {
+        const int Y = i / G, x4 = 4 * (i % G);
+        const uint32_t *rows[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            rows[k] = reinterpret_cast<const uint32_t *>(s + refl101(2 * Y + k - 2, h) * S) + x4 / 2;
+        uint32_t sl[4], sh[4];  // columns 2 x4 - 4 .. 2 x4 + 11
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            uint32_t v[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) v[k] = rows[k][c];
+            vsum4(v, sl[c], sh[c]);
+        }
+        const uint32_t p[6] = {__byte_perm(sl[0], sh[0], 0x7632), __byte_perm(sl[1], sh[1], 0x5410),
+                               __byte_perm(sl[1], sh[1], 0x7632), __byte_perm(sl[2], sh[2], 0x5410),
+                               __byte_perm(sl[2], sh[2], 0x7632), __byte_perm(sl[3], sh[3], 0x5410)};
+        const uint32_t o = hsum4(p);
+        *reinterpret_cast<uint32_t *>(d + Y * D + 4 + x4) = o;
+        store_px4(g + (size_t)Y * gpitch, x4, W, o);
+    }
+    __syncwarp();
+}
+
+// The tail of a frame's pyramid: the levels from c (the first level of at most
+// kTailMaxPx bytes) down to the last, with their Scharr planes, from level c
+// held in shared memory.  Part 0 of `parts` builds the levels below c; the
+// others write row bands of level c's planes (part 0 writes them itself when
+// it is alone).  Level c comes from the tiled launches, or for c = 0 from the
+// caller's image (part 0 then writes the level-0 copy).  A last level too
+// large for shared memory (a large pyramid of few levels) gets its Scharr
+// planes tile by tile from global memory.
+//
+// Bound by the latency of its chain of small levels (a barrier each); four
+// pixels a thread with the tile kernel's packed arithmetic instead of 25 byte
+// reads a pixel, and the bands load only their rows: 18.3 -> 12.4 us for one
+// 960 x 600 frame of 5 levels, 25.0 -> 17.8 us for 32 frames (cold caches).
+template <int GT>
+__device__ __forceinline__ void tail_build(const Level *lv, int levels, int c, int part, int parts, const uint8_t *img,
+                                           int pitch, bool vec_ok, uint8_t *smem) {
+    const Level Lc = lv[c];
+    const uint8_t *src = c == 0 ? img : Lc.img;
+    const int sp = c == 0 ? pitch : Lc.pitch, w = Lc.w, h = Lc.h;
+    if (tail_fits(Lc)) {
+        uint8_t *cur = smem, *nxt = smem + TAIL_A;
+        const int bands = parts > 1 ? parts - 1 : 1, band = (h + bands - 1) / bands;
+        const int y0 = (parts > 1 ? part - 1 : 0) * band, y1 = min(h, y0 + band);  // this part's band (part 0 of many: none)
+        const bool chain = part == 0;
+        if (!chain && (GT == VT_GRAD_NONE || y0 >= y1)) return;
+        const int r0 = chain ? 0 : max(0, y0 - 1), r1 = chain ? h : min(h, y1 + 1);  // rows needed
+        const int S = tail_stride(w);
+        if (c > 0) {  // a pyramid level: 16-byte aligned rows
+            const int C = (w + 15) / 16;
+            for (int i = threadIdx.x; i < (r1 - r0) * C; i += blockDim.x) {
+                const int y = r0 + i / C, k = i % C;
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(Lc.img + (size_t)y * Lc.pitch) + k);
+                uint32_t *d = reinterpret_cast<uint32_t *>(cur + y * S) + 1 + 4 * k;
+                const int room = S / 4 - 1 - 4 * k;  // words left in the row
+                if (room > 0) d[0] = v.x;
+                if (room > 1) d[1] = v.y;
+                if (room > 2) d[2] = v.z;
+                if (room > 3) d[3] = v.w;
+            }
+        } else {  // the caller's image: any alignment
+            const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+            for (int y = r0 + (threadIdx.x >> 5); y < r1; y += nw) {
+                const uint8_t *sr = src + (size_t)y * sp;
+                for (int x = lane; x < w; x += 32) {
+                    const uint8_t v = sr[x];
+                    cur[y * S + 4 + x] = v;
+                    if (chain && src != Lc.img) Lc.img[(size_t)y * Lc.pitch + x] = v;
+                }
+            }
+        }
+        __syncwarp();
+        __syncthreads();
+        tail_pad(cur, w, r0, r1);
+        __syncthreads();
+        if constexpr (GT != VT_GRAD_NONE)
+            if (!chain || parts == 1) tail_scharr<GT>(cur, w, h, y0, y1, Lc.grad, Lc.gpitch);
+        if (!chain) return;
+        for (int l = c; l + 1 < levels; ++l) {
+            const int lw = lv[l].w, lh = lv[l].h;
+            const Level N = lv[l + 1];
+            tail_pyrdown(cur, lw, lh, nxt, N.img, N.pitch);
+            __syncthreads();
+            tail_pad(nxt, N.w, 0, N.h);
+            __syncthreads();
+            if constexpr (GT != VT_GRAD_NONE) tail_scharr<GT>(nxt, N.w, N.h, 0, N.h, N.grad, N.gpitch);
+            uint8_t *t = cur;
+            cur = nxt;
+            nxt = t;
+        }
+    } else if constexpr (GT != VT_GRAD_NONE) {
+        uint8_t (*s_in)[SC_IW] = reinterpret_cast<uint8_t (*)[SC_IW]>(smem);
+        int tiles_x;
+        const int tiles = scharr_tiles(w, h, tiles_x);
+        for (int t = part; t < tiles; t += parts) {
+            const int ty = t / tiles_x, tx = t - ty * tiles_x;
+            scharr_tile<GT>(src, w, h, sp, c == 0 ? vec_ok : true, Lc.grad, Lc.gpitch,
+                            (c == 0 && src != Lc.img) ? Lc.img : nullptr, Lc.pitch, tx, ty, s_in);
+        }
+    } else if (c == 0 && src != Lc.img) {  // no gradients: only the level-0 copy of a large one-level pyramid
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int y = part * nw + (threadIdx.x >> 5); y < h; y += parts * nw)
+            for (int x = lane; x < w; x += 32) Lc.img[(size_t)y * Lc.pitch + x] = src[(size_t)y * sp + x];
     }
 }
 
-// The tail of each frame's pyramid: the levels from c (the first level of at
-// most kTailMaxPx pixels) down to the last, with their Scharr planes, from
-// level c held in shared memory.  A frame's tail is split in `parts` row
-// bands of level c's gradients, one CTA each; part 0 also builds the levels
-// below c.  Level c comes from the tiled launches, or for c = 0 from the
-// caller's image (part 0 then writes the level-0 copy).  A last level too
-// large for shared memory (a large one-level pyramid) gets its Scharr planes
-// tile by tile from global memory.
+// The tails of a batch: every part of every frame (the jobs of the tail list).
 template <int GT>
 __global__ void __launch_bounds__(TAIL_THREADS) k_pyr_tail(const uint8_t *tab) {
     extern __shared__ __align__(16) uint8_t tail_smem[];
@@ -549,63 +705,7 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_pyr_tail(const uint8_t *tab) {
         if (j + (int)gridDim.x >= njobs) pdl_trigger();  // this CTA's last job
         const BLvlJob jb = jobs[j];
         const BFrame fr = frames[jb.frame];
-        const int c = jb.aux;
-        const int part = jb.tiles_x, parts = jb.tile0;  // tail lists: band index and band count
-        const Level Lc = fr.lv[c];
-        const uint8_t *src = c == 0 ? fr.img : Lc.img;
-        const int sp = c == 0 ? fr.pitch : Lc.pitch;
-        if ((long)Lc.pitch * Lc.h <= kTailMaxPx) {
-            // level c in shared memory with the pyramid's row pitch
-            uint8_t *cur = tail_smem, *nxt = tail_smem + TAIL_A;
-            if (c > 0) {  // a pyramid level: 16-byte aligned rows
-                const int n16 = Lc.pitch * Lc.h / 16;
-                const uint4 *g4 = reinterpret_cast<const uint4 *>(Lc.img);
-                uint4 *s4 = reinterpret_cast<uint4 *>(cur);
-                for (int i = threadIdx.x; i < n16; i += blockDim.x) s4[i] = __ldg(g4 + i);
-            } else {  // the caller's image: any alignment
-                const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-                for (int y = threadIdx.x >> 5; y < Lc.h; y += nw) {
-                    const uint8_t *sr = src + (size_t)y * sp;
-                    for (int x = lane; x < Lc.w; x += 32) {
-                        const uint8_t v = sr[x];
-                        cur[y * Lc.pitch + x] = v;
-                        if (part == 0 && src != Lc.img) Lc.img[(size_t)y * Lc.pitch + x] = v;
-                    }
-                }
-            }
-            __syncthreads();
-            const int band = (Lc.h + parts - 1) / parts;
-            const int y0 = part * band, y1 = min(Lc.h, y0 + band);
-            if constexpr (GT != VT_GRAD_NONE) tail_scharr<GT>(cur, Lc.pitch, Lc.w, Lc.h, y0, y1, Lc.grad, Lc.gpitch);
-            if (part == 0) {
-                int stride = Lc.pitch;
-                for (int l = c; l + 1 < fr.levels; ++l) {
-                    const Level L = fr.lv[l], N = fr.lv[l + 1];
-                    tail_pyrdown(cur, stride, L.w, L.h, nxt, N.img, N.pitch);
-                    __syncthreads();
-                    if constexpr (GT != VT_GRAD_NONE) tail_scharr<GT>(nxt, N.w, N.w, N.h, 0, N.h, N.grad, N.gpitch);
-                    uint8_t *t = cur;
-                    cur = nxt;
-                    nxt = t;
-                    stride = N.w;
-                }
-            }
-        } else if (part == 0) {
-            if constexpr (GT != VT_GRAD_NONE) {
-                uint8_t (*s_in)[SC_IW] = reinterpret_cast<uint8_t (*)[SC_IW]>(tail_smem);
-                int tiles_x;
-                const int tiles = scharr_tiles(Lc.w, Lc.h, tiles_x);
-                for (int t = 0; t < tiles; ++t) {
-                    const int ty = t / tiles_x, tx = t - ty * tiles_x;
-                    scharr_tile<GT>(src, Lc.w, Lc.h, sp, c == 0 ? fr.vec_ok != 0 : true, Lc.grad, Lc.gpitch,
-                                    (c == 0 && src != Lc.img) ? Lc.img : nullptr, Lc.pitch, tx, ty, s_in);
-                }
-            } else if (c == 0 && src != Lc.img) {  // no gradients: only the level-0 copy of a large one-level pyramid
-                const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-                for (int y = threadIdx.x >> 5; y < Lc.h; y += nw)
-                    for (int x = lane; x < Lc.w; x += 32) Lc.img[(size_t)y * Lc.pitch + x] = src[(size_t)y * sp + x];
-            }
-        }
+        tail_build<GT>(fr.lv, fr.levels, jb.aux, jb.tiles_x, jb.tile0, fr.img, fr.pitch, fr.vec_ok != 0, tail_smem);
         __syncthreads();
     }
 }
