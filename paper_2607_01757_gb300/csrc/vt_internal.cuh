@@ -81,35 +81,29 @@ inline cudaError_t launch_pdl(void (*k)(Params...), int grid, int block, size_t 
 
 // ---------------------------------------------------------------- pyramid jobs
 // A pyrDown (and optionally Scharr) job: level src (w x h) -> dst
-// (ceil(w/2) x ceil(h/2)); gradients of the src level when grad != nullptr.
+// (ceil(w/2) x ceil(h/2)); gradients of the src level in the variants with
+// them; the src level copied to `copy` when it is not null.
 struct PyrJob {
     const uint8_t *src;
-    uint8_t *dst;
+    uint8_t *dst, *copy;
     uint32_t *grad;
-    int w, h, spitch, dpitch, gpitch;
+    int w, h, spitch, dpitch, gpitch, cpitch, vec_ok;
     int tiles_x;  // output tiles along x
-    int tile0;    // first block of this job
 };
 
-constexpr int kMaxJobs = 48;
-
-struct PyrJobs {
-    int njobs;
-    PyrJob j[kMaxJobs];
-};
-
-// A Scharr-only job over one level.
+// A Scharr-only job over one level (copied to `copy` when it is not null).
 struct GradJob {
     const uint8_t *src;
     uint32_t *grad;
-    int w, h, spitch, gpitch;
+    uint8_t *copy;
+    int w, h, spitch, gpitch, cpitch, vec_ok;
     int tiles_x;
     int tile0;
 };
 
 struct GradJobs {
     int njobs;
-    GradJob j[kMaxJobs];
+    GradJob j[VT_MAX_LEVELS];
 };
 
 // Tracking parameters as the kernels use them.
@@ -219,9 +213,5 @@ int pyr_batch_blocks_per_sm();
 int pyr_tiles(int w, int h, int &tiles_x);
 __host__ __device__ int scharr_tiles(int w, int h, int &tiles_x);
 bool window_supported(int win);
-vt_status launch_pyrdown(const PyrJobs &jobs, int total_blocks, int gtype, cudaStream_t s);
-vt_status launch_scharr(const GradJobs &jobs, int total_blocks, int gtype, cudaStream_t s);
-void add_pyr_job(PyrJobs &jobs, int &blocks, const Level &src, const Level &dst, bool with_grad);
-void add_grad_job(GradJobs &jobs, int &blocks, const Level &lv);
 
 }  // namespace vt

@@ -9,11 +9,10 @@
 // Table I); these are the readings implemented.
 //
 // Layout: a CTA stages its input tile (plus halo) in shared memory with
-// 16-byte vector loads when the tile is inside the image, or with
-// reflect-101 index mapping byte by byte on border tiles.  The same staged
-// tile serves the pyramid step and, in the fused variant, the gradients of
-// the source level.  Several levels / frames run in one launch through a
-// job table passed as a __grid_constant__ kernel parameter.
+// 16-byte loads, the reflected columns of edge tiles filled in afterwards.
+// The same staged tile serves the pyramid step and, in the fused variant, the
+// gradients of the source level and the copy of a caller's frame.  A frame's
+// small levels are built together from shared memory (tail_build).
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -399,28 +398,29 @@ __device__ __forceinline__ void scharr_tile(const uint8_t *src, int w, int h, in
     __syncthreads();
 }
 
+// One level of one frame (level 0 may come from the caller's image, with the
+// level-0 copy written from the same tile).
 template <bool GRAD, int GT>
-__global__ void __launch_bounds__(PD_THREADS) k_pyrdown(const __grid_constant__ PyrJobs J) {
+__global__ void __launch_bounds__(PD_THREADS) k_pyrdown(const __grid_constant__ PyrJob J) {
     __shared__ __align__(16) uint8_t s_in[PD_IH][PD_IW];
     __shared__ uint16_t s_v[PD_TH][PD_VW];
-    int k = 0;
-    while (k + 1 < J.njobs && (int)blockIdx.x >= J.j[k + 1].tile0) ++k;
-    const PyrJob &jb = J.j[k];
-    const int t = blockIdx.x - jb.tile0;
-    const int ty = t / jb.tiles_x, tx = t - ty * jb.tiles_x;
-    pyr_tile<GRAD, GT>(jb.src, jb.w, jb.h, jb.spitch, true, jb.dst, jb.dpitch, jb.grad, jb.gpitch, nullptr, 0, tx,
-                       ty, s_in, s_v);
+    pdl_wait();  // the level (or the caller's image) is the previous launch's output
+    pdl_trigger();
+    const int ty = blockIdx.x / J.tiles_x, tx = blockIdx.x - ty * J.tiles_x;
+    pyr_tile<GRAD, GT>(J.src, J.w, J.h, J.spitch, J.vec_ok != 0, J.dst, J.dpitch, J.grad, J.gpitch, J.copy, J.cpitch,
+                       tx, ty, s_in, s_v);
 }
 
 template <int GT>
 __global__ void __launch_bounds__(SC_THREADS) k_scharr(const __grid_constant__ GradJobs J) {
     __shared__ __align__(16) uint8_t s_in[SC_IH][SC_IW];
+    pdl_wait();
     int k = 0;
     while (k + 1 < J.njobs && (int)blockIdx.x >= J.j[k + 1].tile0) ++k;
     const GradJob &jb = J.j[k];
     const int t = blockIdx.x - jb.tile0;
     const int ty = t / jb.tiles_x, tx = t - ty * jb.tiles_x;
-    scharr_tile<GT>(jb.src, jb.w, jb.h, jb.spitch, true, jb.grad, jb.gpitch, nullptr, 0, tx, ty, s_in);
+    scharr_tile<GT>(jb.src, jb.w, jb.h, jb.spitch, jb.vec_ok != 0, jb.grad, jb.gpitch, jb.copy, jb.cpitch, tx, ty, s_in);
 }
 
 // --------------------------------------------------------- batched (persistent)
@@ -710,6 +710,20 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_pyr_tail(const uint8_t *tab) {
     }
 }
 
+// The tail of one frame's pyramid (one CTA per part).
+struct TailArgs {
+    Level lv[VT_MAX_LEVELS];
+    int levels, c, pitch, vec_ok;
+    const uint8_t *img;
+};
+
+template <int GT>
+__global__ void __launch_bounds__(TAIL_THREADS) k_pyr_tail_one(const __grid_constant__ TailArgs A) {
+    extern __shared__ __align__(16) uint8_t tail_smem[];
+    pdl_wait();
+    tail_build<GT>(A.lv, A.levels, A.c, blockIdx.x, gridDim.x, A.img, A.pitch, A.vec_ok != 0, tail_smem);
+}
+
 int pyr_tiles(int w, int h, int &tiles_x) {
     const int W = (w + 1) / 2, H = (h + 1) / 2;
     tiles_x = (W + PD_TW - 1) / PD_TW;
@@ -721,16 +735,15 @@ __host__ __device__ int scharr_tiles(int w, int h, int &tiles_x) {
     return tiles_x * ((h + SC_TH - 1) / SC_TH);
 }
 
+template <typename K>
+static bool tail_smem_ok(K *k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM) == cudaSuccess;
+}
+
 vt_status launch_pyr_batch(const uint8_t *dev_tab, int tiled_launches, int gtype, int grid_pyr, int grid_tail,
                            cudaStream_t s, cudaEvent_t *ev) {
-    static const bool attr = [] {  // once, thread-safe static initialisation
-        return cudaFuncSetAttribute(k_pyr_tail<VT_GRAD_S16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TAIL_SMEM) == cudaSuccess &&
-               cudaFuncSetAttribute(k_pyr_tail<VT_GRAD_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TAIL_SMEM) == cudaSuccess &&
-               cudaFuncSetAttribute(k_pyr_tail<VT_GRAD_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TAIL_SMEM) == cudaSuccess;
-    }();
+    static const bool attr = tail_smem_ok(k_pyr_tail<VT_GRAD_S16>) && tail_smem_ok(k_pyr_tail<VT_GRAD_F16>) &&
+                             tail_smem_ok(k_pyr_tail<VT_GRAD_NONE>);  // once, thread-safe static initialisation
     (void)attr;
     // every launch after the first overlaps its start with the previous one's
     // end (programmatic dependent launch), except where an event is recorded
@@ -755,56 +768,33 @@ int pyr_batch_blocks_per_sm() {
     return a;
 }
 
-void add_pyr_job(PyrJobs &jobs, int &blocks, const Level &src, const Level &dst, bool with_grad) {
-    PyrJob &j = jobs.j[jobs.njobs++];
-    j.src = src.img;
-    j.dst = dst.img;
-    j.grad = with_grad ? src.grad : nullptr;
-    j.w = src.w;
-    j.h = src.h;
-    j.spitch = src.pitch;
-    j.dpitch = dst.pitch;
-    j.gpitch = src.gpitch;
-    const int W = (src.w + 1) / 2, H = (src.h + 1) / 2;
-    j.tiles_x = (W + PD_TW - 1) / PD_TW;
-    const int tiles_y = (H + PD_TH - 1) / PD_TH;
-    j.tile0 = blocks;
-    blocks += j.tiles_x * tiles_y;
-}
-
-void add_grad_job(GradJobs &jobs, int &blocks, const Level &lv) {
+// A Scharr job over level `lv`, read from `src` (the level itself, or the
+// caller's image, then also copied to the level).
+static void add_grad_job(GradJobs &jobs, int &blocks, const Level &lv, const uint8_t *src, int spitch, int vec_ok) {
     GradJob &j = jobs.j[jobs.njobs++];
-    j.src = lv.img;
+    j.src = src;
     j.grad = lv.grad;
+    j.copy = src != lv.img ? lv.img : nullptr;
     j.w = lv.w;
     j.h = lv.h;
-    j.spitch = lv.pitch;
+    j.spitch = spitch;
     j.gpitch = lv.gpitch;
-    j.tiles_x = (lv.w + SC_TW - 1) / SC_TW;
-    const int tiles_y = (lv.h + SC_TH - 1) / SC_TH;
+    j.cpitch = lv.pitch;
+    j.vec_ok = vec_ok;
     j.tile0 = blocks;
-    blocks += j.tiles_x * tiles_y;
+    blocks += scharr_tiles(lv.w, lv.h, j.tiles_x);
 }
 
-vt_status launch_pyrdown(const PyrJobs &jobs, int total_blocks, int gtype, cudaStream_t s) {
+// Every launch of a build starts while the stream's previous kernel ends
+// (programmatic dependent launch): a build is a chain of launches of a few
+// microseconds each, and the launch latency between them cost as much as the
+// kernels.
+static vt_status launch_scharr(const GradJobs &jobs, int total_blocks, int gtype, cudaStream_t s) {
     if (jobs.njobs == 0 || total_blocks == 0) return VT_OK;
-    const bool grad = jobs.j[0].grad != nullptr;
-    if (!grad)
-        k_pyrdown<false, VT_GRAD_S16><<<total_blocks, PD_THREADS, 0, s>>>(jobs);
-    else if (gtype == VT_GRAD_F16)
-        k_pyrdown<true, VT_GRAD_F16><<<total_blocks, PD_THREADS, 0, s>>>(jobs);
-    else
-        k_pyrdown<true, VT_GRAD_S16><<<total_blocks, PD_THREADS, 0, s>>>(jobs);
-    return cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
-}
-
-vt_status launch_scharr(const GradJobs &jobs, int total_blocks, int gtype, cudaStream_t s) {
-    if (jobs.njobs == 0 || total_blocks == 0) return VT_OK;
-    if (gtype == VT_GRAD_F16)
-        k_scharr<VT_GRAD_F16><<<total_blocks, SC_THREADS, 0, s>>>(jobs);
-    else
-        k_scharr<VT_GRAD_S16><<<total_blocks, SC_THREADS, 0, s>>>(jobs);
-    return cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
+    return launch_pdl(gtype == VT_GRAD_F16 ? k_scharr<VT_GRAD_F16> : k_scharr<VT_GRAD_S16>, total_blocks, SC_THREADS, 0,
+                      s, true, jobs) == cudaSuccess
+               ? VT_OK
+               : VT_ERR_CUDA;
 }
 
 // ------------------------------------------------------------------ host side
@@ -870,6 +860,20 @@ static vt_status check_build_args(const uint8_t *img, int w, int h, int pitch, i
     return VT_OK;
 }
 
+// Whether a kernel on the current device may read `p` as it is: its own
+// memory, managed or pinned host memory (anything else is left to the copy
+// call, which reaches other devices and refuses what it cannot read).
+static bool kernel_readable(const void *p) {
+    cudaPointerAttributes a;
+    int dev = 0;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || a.type == cudaMemoryTypeHost ||
+           (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int levels, int img_on_device, int gtype,
                             void *cuda_stream, vt_pyramid **out) {
     vt_status st = check_build_args(img, w, h, pitch, levels, out);
@@ -884,34 +888,71 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const Level &L0 = p->lv[0];
     if (img == L0.img && pitch != L0.pitch) return VT_ERR_ARG;
-    // a frame already in level 0 (vt_pyramid_upload) is built in place
-    cudaError_t e = img == L0.img ? cudaSuccess
-                                  : cudaMemcpy2DAsync(L0.img, L0.pitch, img, pitch, w, h,
-                                                      img_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) {
+    const bool grad = gtype != VT_GRAD_NONE;
+    const int c = tail_start_level(p);
+    const bool small = tail_fits(p->lv[c]);  // the levels from c on take one launch
+    // A frame already in level 0 (vt_pyramid_upload) is built in place, and a
+    // device image is copied by the launch that reads it first; host images
+    // (and one-level pyramids without planes) are copied up first.
+    const bool by_kernel = img_on_device && img != L0.img && (c > 0 || small || grad) && kernel_readable(img);
+    cudaError_t e = cudaSuccess;
+    if (img != L0.img && !by_kernel) {
+        e = cudaMemcpy2DAsync(L0.img, L0.pitch, img, pitch, w, h,
+                              img_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
+        img = L0.img;
+        pitch = L0.pitch;
+    }
+    const int vec_ok = (uintptr_t)img % 16 == 0 && pitch % 16 == 0;
+    for (int l = 0; l < c && e == cudaSuccess; ++l) {
+        const Level &S = p->lv[l], &D = p->lv[l + 1];
+        PyrJob j;
+        j.src = l == 0 ? img : S.img;
+        j.spitch = l == 0 ? pitch : S.pitch;
+        j.vec_ok = l == 0 ? vec_ok : 1;
+        j.copy = j.src != S.img ? S.img : nullptr;
+        j.cpitch = S.pitch;
+        j.dst = D.img;
+        j.dpitch = D.pitch;
+        j.grad = S.grad;
+        j.gpitch = S.gpitch;
+        j.w = S.w;
+        j.h = S.h;
+        const int tiles = pyr_tiles(S.w, S.h, j.tiles_x);
+        e = launch_pdl(!grad                    ? k_pyrdown<false, VT_GRAD_S16>
+                       : gtype == VT_GRAD_F16 ? k_pyrdown<true, VT_GRAD_F16>
+                                              : k_pyrdown<true, VT_GRAD_S16>,
+                       tiles, PD_THREADS, 0, s, true, j);
+    }
+    if (e == cudaSuccess && small) {
+        static const bool attr = tail_smem_ok(k_pyr_tail_one<VT_GRAD_S16>) && tail_smem_ok(k_pyr_tail_one<VT_GRAD_F16>) &&
+                                 tail_smem_ok(k_pyr_tail_one<VT_GRAD_NONE>);  // once, thread-safe static initialisation
+        (void)attr;
+        TailArgs A;
+        for (int l = 0; l < VT_MAX_LEVELS; ++l) A.lv[l] = l < levels ? p->lv[l] : Level{};
+        A.levels = levels;
+        A.c = c;
+        A.img = img;
+        A.pitch = pitch;
+        A.vec_ok = vec_ok;
+        e = launch_pdl(!grad                    ? k_pyr_tail_one<VT_GRAD_NONE>
+                       : gtype == VT_GRAD_F16 ? k_pyr_tail_one<VT_GRAD_F16>
+                                              : k_pyr_tail_one<VT_GRAD_S16>,
+                       grad ? tail_parts(p) : 1, TAIL_THREADS, TAIL_SMEM, s, true, A);
+    } else if (e == cudaSuccess && grad) {  // (c is the last level)
+        GradJobs gj;
+        gj.njobs = 0;
+        int blocks = 0;
+        add_grad_job(gj, blocks, p->lv[c], c == 0 ? img : p->lv[c].img, c == 0 ? pitch : p->lv[c].pitch,
+                     c == 0 ? vec_ok : 1);
+        if (launch_scharr(gj, blocks, gtype, s) != VT_OK) e = cudaErrorLaunchFailure;
+    }
+    if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         cudaGetLastError();
         if (fresh) {
             vt_pyramid_free(p);
             *out = nullptr;
         }
         return VT_ERR_CUDA;
-    }
-    const bool grad = gtype != VT_GRAD_NONE;
-    for (int l = 0; l + 1 < levels; ++l) {
-        PyrJobs jobs;
-        jobs.njobs = 0;
-        int blocks = 0;
-        add_pyr_job(jobs, blocks, p->lv[l], p->lv[l + 1], grad);
-        st = launch_pyrdown(jobs, blocks, gtype, s);
-        if (st != VT_OK) return st;
-    }
-    if (grad) {
-        GradJobs gj;
-        gj.njobs = 0;
-        int blocks = 0;
-        add_grad_job(gj, blocks, p->lv[levels - 1]);
-        st = launch_scharr(gj, blocks, gtype, s);
-        if (st != VT_OK) return st;
     }
     p->gtype = grad ? gtype : VT_GRAD_NONE;
     return VT_OK;
@@ -939,8 +980,8 @@ vt_status vt_gradients(vt_pyramid *p, vt_grad_type t, void *cuda_stream) {
     GradJobs gj;
     gj.njobs = 0;
     int blocks = 0;
-    for (int l = 0; l < p->levels; ++l) add_grad_job(gj, blocks, p->lv[l]);
-    vt_status st = launch_scharr(gj, blocks, (int)t, (cudaStream_t)cuda_stream);
+    for (int l = 0; l < p->levels; ++l) add_grad_job(gj, blocks, p->lv[l], p->lv[l].img, p->lv[l].pitch, 1);
+    const vt_status st = launch_scharr(gj, blocks, (int)t, (cudaStream_t)cuda_stream);
     if (st == VT_OK) p->gtype = (int)t;
     return st;
 }
