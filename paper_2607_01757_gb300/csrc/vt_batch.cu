@@ -220,7 +220,6 @@ struct vt_batch {
     int klt_ctas_per_sm;  // 0 = occupancy limit
     int pyr_grid;
     int tail_grid;  // CTAs of the tail launch (one frame each at a time)
-    int gate_grid;  // CTAs of the stereo-gate launch
 };
 
 namespace vt {
@@ -280,7 +279,7 @@ static vt_status enqueue(vt_batch *b, int k, cudaStream_t s, cudaEvent_t *ev = n
     if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return VT_ERR_CUDA;
     if (tp.fp64 && launch_klt_f64(b->dev[k], tp.win, tp.gtype, b->sms * 4, s) != VT_OK) return VT_ERR_CUDA;
     if (ev && ev[3]) cudaEventRecord(ev[3], s);
-    if (tp.gate) return launch_gate_batch(b->dev[k], b->gate_grid, s);
+    if (tp.gate) return launch_gate_batch(b->dev[k], b->sms, !ev, s);
     return VT_OK;
 }
 
@@ -316,7 +315,6 @@ vt_status vt_batch_create(int max_frames, int max_tasks, vt_batch **out) {
     b->klt_ctas_per_sm = 0;
     b->tail_grid = 8 * b->cap_frames < 2 * b->sms ? 8 * b->cap_frames : 2 * b->sms;
     b->pyr_grid = b->sms * (pyr_batch_blocks_per_sm() > 0 ? pyr_batch_blocks_per_sm() : 1);
-    b->gate_grid = 4 * b->sms;
     b->staged = -1;
     *out = b;
     return VT_OK;
@@ -525,6 +523,8 @@ vt_status vt_batch_set_gates(vt_batch *b, const vt_gate_task *gates, int ngates,
     for (int i = 0; i < ngates; ++i) {
         const vt_gate_task &g = gates[i];
         gt[i].rig = g.rig;
+        gt[i].inv[0] = 1.0 / g.rig.kl[0], gt[i].inv[1] = 1.0 / g.rig.kl[1];
+        gt[i].inv[2] = 1.0 / g.rig.kr[0], gt[i].inv[3] = 1.0 / g.rig.kr[1];
         gt[i].pts_l = reinterpret_cast<const float2 *>(g.pts_l);
         gt[i].pts_r = reinterpret_cast<const float2 *>(g.pts_r);
         gt[i].status_in = g.status_in;

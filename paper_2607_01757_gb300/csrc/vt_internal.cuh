@@ -179,6 +179,7 @@ struct BTask {
 // One stereo-gate task of a batched run: a rig and the pairs it checks.
 struct GTask {
     vt_stereo_rig rig;
+    double inv[4];  // 1 / fx, 1 / fy of the left and the right camera
     const float2 *pts_l, *pts_r;
     const uint8_t *status_in;
     float *xyz;
@@ -199,8 +200,8 @@ struct BatchHdr {
 };
 
 // Batched stereo gate (vt_stereo.cu): every gate task of the table at dev_tab,
-// grid-stride over their pairs.
-vt_status launch_gate_batch(const uint8_t *dev_tab, int grid, cudaStream_t s);
+// grid-stride over their pairs (pdl: as a dependent of the launch before).
+vt_status launch_gate_batch(const uint8_t *dev_tab, int sms, bool pdl, cudaStream_t s);
 bool gate_args_ok(const vt_stereo_rig *rig, const vt_gate_params *prm);
 
 // Host helpers implemented in vt_pyramid.cu.
