@@ -399,6 +399,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
     H->P.min_eig = prm->min_eig;
     H->P.fb_thr2 = prm->fb_thr * prm->fb_thr;
     H->P.fp64 = fp64_needed(prm->min_eig);
+    H->P.want_lmin = 0;
     BFrame *bf = reinterpret_cast<BFrame *>(tab + H->off_frames);
     BLvlJob *jobs = reinterpret_cast<BLvlJob *>(tab + H->off_jobs);
     BTileSrc *tsrc = reinterpret_cast<BTileSrc *>(tab + H->off_tsrc);
@@ -788,6 +789,7 @@ extern "C" vt_status vt_klt_track_tasks_noalloc(const vt_track_task *tasks, int 
     H->P.min_eig = prm->min_eig;
     H->P.fb_thr2 = prm->fb_thr * prm->fb_thr;
     H->P.fp64 = fp64_needed(prm->min_eig);
+    H->P.want_lmin = 0;
     int p0 = 0;
     for (int t = 0; t < ntasks; ++t) {
         const vt_track_task &tk = tasks[t];

@@ -112,6 +112,7 @@ struct KParams {
     float eps2;     // eps^2
     float min_eig;  // threshold on lambda_min / (win^2 255^2)
     float fb_thr2;  // fb_thr^2
+    int want_lmin;  // the caller reads lambda_min
     int fp64;       // ill-conditioned levels go to the FP64-capable launch (see fp64_needed)
 };
 

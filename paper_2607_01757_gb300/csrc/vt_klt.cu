@@ -141,6 +141,7 @@ static vt_status track_common(const vt_pyramid *prev, const vt_pyramid *cur, con
     A.P.min_eig = prm->min_eig;
     A.P.fb_thr2 = prm->fb_thr * prm->fb_thr;
     A.P.fp64 = fp64_needed(prm->min_eig);
+    A.P.want_lmin = A.lmin != nullptr;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (prev->gtype == VT_GRAD_F16)
         return fb ? dispatch_win<VT_GRAD_F16, true>(A, s) : dispatch_win<VT_GRAD_F16, false>(A, s);

@@ -426,15 +426,18 @@ __device__ __forceinline__ void run_columns(int x0, int w, int sx, int c, int &o
     }
 }
 
-// The template at the lane's window samples (KRuns): T (times 2^-22, see px) and its gradients,
+// The template at the lane's window samples (KRuns): N = -T (times 2^-22, see
+// px) and its gradients,
 // sampled at fractional offset (ax, ay) from the staged windows, zero for
 // samples outside the window.
 template <int WIN, int GT>
 __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const TWin &W, float ax, float ay, int lane,
-                                                float (&T)[KRuns<WIN>::NS], float2 (&G)[KRuns<WIN>::NS]) {
+                                                float (&N)[KRuns<WIN>::NS], float2 (&G)[KRuns<WIN>::NS]) {
     constexpr int TS = twin_stride<WIN, GT>(), GS = KSmem<WIN>::GS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
     // staged gradient words are int16 pairs when computed in place
     constexpr int GTS = GT == VT_GRAD_NONE ? VT_GRAD_S16 : GT;
+    const uint8_t *j0[RPL], *j1[RPL];
+    const uint32_t *g0[RPL], *g1[RPL];
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
         int c, r0;
@@ -442,24 +445,42 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const TWin &
         run_of<WIN>(lane, i, c, r0, valid);
         int o0, o1;
         run_columns<WIN>(W.x0, W.w, W.sx, c, o0, o1);
-        const uint8_t *j0 = valid ? W.st + r0 * TS + o0 : C.zj, *j1 = valid ? W.st + r0 * TS + o1 : C.zj;
+        j0[i] = valid ? W.st + r0 * TS + o0 : C.zj, j1[i] = valid ? W.st + r0 * TS + o1 : C.zj;
         run_columns<WIN>(W.gx0, W.gw, W.gsx, c, o0, o1);
-        const uint32_t *g0 = valid ? W.sg + r0 * GS + o0 : C.zg, *g1 = valid ? W.sg + r0 * GS + o1 : C.zg;
-        float pi = 0.f;
+        g0[i] = valid ? W.sg + r0 * GS + o0 : C.zg, g1[i] = valid ? W.sg + r0 * GS + o1 : C.zg;
+    }
+    // the image, a lane's two runs as a pair (a lone run's second half is idle)
+    float2 pt = pair(0.f);
+#pragma unroll
+    for (int r = 0; r <= RL; ++r) {
+        const float2 l = make_float2(__uint_as_float(j0[0][r * TS]), __uint_as_float(j0[RPL - 1][r * TS]));
+        const float2 n = make_float2(__uint_as_float(j1[0][r * TS]), __uint_as_float(j1[RPL - 1][r * TS]));
+        float2 nh;  // minus the horizontal lerp
+        if constexpr (RPL == 2) {
+            const float2 nl = __fmul2_rn(l, pair(-px_scale()));
+            nh = __ffma2_rn(pair(-ax), __ffma2_rn(n, pair(px_scale()), nl), nl);
+            if (r > 0) {
+                const float2 t = __ffma2_rn(pair(ay), sub2(nh, pt), pt);
+                N[r - 1] = t.x, N[RL + r - 1] = t.y;  // zero for a run outside the window
+            }
+        } else {
+            const float nl = l.x * -px_scale();
+            nh.x = fmaf(-ax, fmaf(n.x, px_scale(), nl), nl);
+            nh.y = 0.f;
+            if (r > 0) N[r - 1] = fmaf(ay, nh.x - pt.x, pt.x);
+        }
+        pt = nh;
+    }
+#pragma unroll
+    for (int i = 0; i < RPL; ++i) {
         float2 pg = pair(0.f);
 #pragma unroll
         for (int r = 0; r <= RL; ++r) {
-            const float mv = px(j0[r * TS]);
             float2 gl, gr;
-            unpack_grad<GTS>(g0[r * GS], gl.x, gl.y);
-            unpack_grad<GTS>(g1[r * GS], gr.x, gr.y);
-            const float hi = fmaf(ax, px_minus(j1[r * TS], mv), mv);
+            unpack_grad<GTS>(g0[i][r * GS], gl.x, gl.y);
+            unpack_grad<GTS>(g1[i][r * GS], gr.x, gr.y);
             const float2 hg = __ffma2_rn(pair(ax), sub2(gr, gl), gl);
-            if (r > 0) {
-                T[i * RL + r - 1] = fmaf(ay, hi - pi, pi);  // zero for a run outside the window
-                G[i * RL + r - 1] = __ffma2_rn(pair(ay), sub2(hg, pg), pg);
-            }
-            pi = hi;
+            if (r > 0) G[i * RL + r - 1] = __ffma2_rn(pair(ay), sub2(hg, pg), pg);
             pg = hg;
         }
     }
@@ -477,7 +498,7 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const TWin &
 // part, y part).  The footprint is staged
 // in sm.j; w: the level's width.
 template <int WIN>
-__device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&T)[KRuns<WIN>::NS],
+__device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&N)[KRuns<WIN>::NS],
                                              const float2 (&G)[KRuns<WIN>::NS], const KSmem<WIN> &sm,
                                              float2 (&m)[4]) {
     constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
@@ -500,7 +521,7 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
             q.y = px_minus(j1[r * JS], q.x);
             if (r > 0) {
                 const int s = i * RL + r - 1;
-                const float e0 = T[s] - p.x;
+                const float e0 = -N[s] - p.x;
                 const float2 d = sub2(q, p);  // F10 - F00, F11 - F10 - F01 + F00
                 a[0] = __ffma2_rn(pair(e0), G[s], a[0]);
                 a[1] = __ffma2_rn(pair(p.y), G[s], a[1]);
@@ -521,9 +542,9 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
 // |T - J(q + x)| over the window.
 template <int WIN>
 __device__ __forceinline__ float abs_residual(const KCta<WIN> &C, int x0, int w, float bx, float by, int lane,
-                                              const float (&T)[KRuns<WIN>::NS], const KSmem<WIN> &sm) {
+                                              const float (&N)[KRuns<WIN>::NS], const KSmem<WIN> &sm) {
     constexpr int JS = KSmem<WIN>::JS, RL = KRuns<WIN>::RL, RPL = KRuns<WIN>::RPL;
-    float sa = 0.f, sb = 0.f;
+    const uint8_t *j0[RPL], *j1[RPL];
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
         int c, r0;
@@ -531,22 +552,34 @@ __device__ __forceinline__ float abs_residual(const KCta<WIN> &C, int x0, int w,
         run_of<WIN>(lane, i, c, r0, valid);
         int o0, o1;
         run_columns<WIN>(x0, w, staged_x(x0, 16), c, o0, o1);
-        const uint8_t *j0 = valid ? &sm.j[r0 * JS + o0] : C.zj, *j1 = valid ? &sm.j[r0 * JS + o1] : C.zj;
-        float ph = 0.f;
+        j0[i] = valid ? &sm.j[r0 * JS + o0] : C.zj, j1[i] = valid ? &sm.j[r0 * JS + o1] : C.zj;
+    }
+    float sa = 0.f, sb = 0.f, later[RL];
+    float2 ph = pair(0.f);
 #pragma unroll
-        for (int r = 0; r <= RL; ++r) {
-            const float mv = px(j0[r * JS]);
-            const float h = fmaf(bx, px_minus(j1[r * JS], mv), mv);
-            if (r > 0) {
-                const float jv = fmaf(by, h - ph, ph);
-                const float e = fabsf(T[i * RL + r - 1] - jv);  // 0 - 0 for a run outside the window
-                if (r & 1)
-                    sa += e;
-                else
-                    sb += e;
-            }
-            ph = h;
+    for (int r = 0; r <= RL; ++r) {
+        const float2 l = make_float2(__uint_as_float(j0[0][r * JS]), __uint_as_float(j0[RPL - 1][r * JS]));
+        const float2 n = make_float2(__uint_as_float(j1[0][r * JS]), __uint_as_float(j1[RPL - 1][r * JS]));
+        const float2 nl = __fmul2_rn(l, pair(-px_scale()));
+        const float2 nh = __ffma2_rn(pair(-bx), __ffma2_rn(n, pair(px_scale()), nl), nl);  // minus the horizontal lerp
+        if (r > 0) {
+            const float2 nj = __ffma2_rn(pair(by), sub2(nh, ph), ph);
+            const float e = fabsf(N[r - 1] - nj.x);  // 0 - 0 for a run outside the window
+            if (r & 1)
+                sa += e;
+            else
+                sb += e;
+            if constexpr (RPL == 2) later[r - 1] = fabsf(N[RL + r - 1] - nj.y);
         }
+        ph = nh;
+    }
+    if constexpr (RPL == 2) {
+#pragma unroll
+        for (int r = 1; r <= RL; ++r)
+            if (r & 1)
+                sa += later[r - 1];
+            else
+                sb += later[r - 1];
     }
     return warp_sum(sa + sb);
 }
@@ -874,15 +907,22 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         }
         float g11, g12, g22;
         warp_sum3(aii.x, a12, aii.y, lane, g11, g12, g22);
-        // lambda_min = det / lambda_max avoids the cancellation of (tr - disc) / 2
         const float tr = g11 + g22, df = g11 - g22;
-        const float lmax = 0.5f * (tr + sqrtf(fmaf(df, df, 4.f * g12 * g12)));
         const float det = kdiff(g11, g22, g12, g12);  // sign exact, 2 ulp
-        const float lmin = det / lmax;
-        o.lmin = lmin * inv_norm;
         nux = nuy = 0.f;
-        // ill-conditioned (or det <= 0): decided and tracked in FP64
-        level64 = P.fp64 && !(lmin * kFp64Cond >= lmax);
+        // lambda_min = det / lambda_max >= det / tr: a template that passes with
+        // that bound by more than the rounding of all this (1e-5 against a few
+        // 1e-7) passes, and the square root and the division are left out
+        // unless the caller wants lambda_min (or a level may need FP64)
+        const bool passes = det * inv_norm > 1.00001f * P.min_eig * tr;
+        if (F64 || P.fp64 || P.want_lmin || !passes) {
+            // det / lambda_max avoids the cancellation of (tr - disc) / 2
+            const float lmax = 0.5f * (tr + sqrtf(fmaf(df, df, 4.f * g12 * g12)));
+            const float lmin = det / lmax;
+            o.lmin = lmin * inv_norm;
+            // ill-conditioned (or det <= 0): decided and tracked in FP64
+            level64 = P.fp64 && !(lmin * kFp64Cond >= lmax);
+        }
         if (level64) {
             if constexpr (!F64) {
                 cp_async_wait<0>();  // nothing may land after the buffers are used again
@@ -913,7 +953,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
                 continue;
             }
         }
-        if (!(o.lmin >= P.min_eig) || !(det > 0.f)) {
+        if (!passes && (!(o.lmin >= P.min_eig) || !(det > 0.f))) {
             o.status = 0;
             o.reason = VT_LOST_EIG;
             lost_level = l;
