@@ -186,9 +186,10 @@ constexpr int kGraphsPerBuffer = 8;
 
 struct Topo {
     int maxL, gtype, win, klt_warps, klt_grid, pyr_grid, gate, fp64;
+    int frames;  // whether the run builds any pyramid
     bool operator==(const Topo &o) const {
         return maxL == o.maxL && gtype == o.gtype && win == o.win && klt_warps == o.klt_warps &&
-               klt_grid == o.klt_grid && pyr_grid == o.pyr_grid && gate == o.gate && fp64 == o.fp64;
+               klt_grid == o.klt_grid && pyr_grid == o.pyr_grid && gate == o.gate && fp64 == o.fp64 && frames == o.frames;
     }
 };
 
@@ -201,7 +202,6 @@ struct vt_batch {
     size_t tab_bytes;
     uint8_t *host[2];
     uint8_t *dev[2];
-    int *counter;  // [2]
     cudaEvent_t ev[2];
     bool ev_used[2];
     int next;    // buffer the next vt_batch_set writes
@@ -260,22 +260,27 @@ static int klt_grid(const vt_batch *b, int win, int gtype) {
 // (nullable): one event after each pyramid launch.
 static vt_status enqueue(vt_batch *b, int k, cudaStream_t s, cudaEvent_t *ev = nullptr, cudaEvent_t *lev = nullptr) {
     const Topo &tp = b->topo[k];
-    if (cudaMemcpyAsync(b->dev[k], b->host[k], b->tab_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(b->counter + k, 0, sizeof(int), s) != cudaSuccess) {
+    // (the work counter is a word of the table: the copy clears it)
+    if (cudaMemcpyAsync(b->dev[k], b->host[k], b->tab_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) {
         cudaGetLastError();
         return VT_ERR_CUDA;
     }
     if (ev && ev[0]) cudaEventRecord(ev[0], s);
-    vt_status st = launch_pyr_batch(b->dev[k], tp.maxL, tp.gtype, tp.pyr_grid, b->tail_grid, s, lev);
-    if (st != VT_OK) return st;
+    if (tp.frames) {
+        const vt_status st = launch_pyr_batch(b->dev[k], tp.maxL, tp.gtype, tp.pyr_grid, b->tail_grid, s, lev);
+        if (st != VT_OK) return st;
+    } else if (lev && lev[0]) {
+        cudaEventRecord(lev[0], s);
+    }
     if (ev && ev[1]) cudaEventRecord(ev[1], s);
     const KltBatchKernel kb = klt_batch_kernel(tp.win, tp.gtype, tp.klt_warps);
     if (!kb.fn) return VT_ERR_ARG;
     if (ev && ev[2]) cudaEventRecord(ev[2], s);
     // starts while the last pyramid launch finishes (programmatic dependent
     // launch), unless events are recorded for per-launch timing
-    const cudaError_t e =
-        launch_pdl(kb.fn, tp.klt_grid, tp.klt_warps * 32, kb.smem, s, !ev, (const uint8_t *)b->dev[k], b->counter + k);
+    const cudaError_t e = launch_pdl(kb.fn, tp.klt_grid, tp.klt_warps * 32, kb.smem, s, !ev && tp.frames,
+                                     (const uint8_t *)b->dev[k],
+                                     reinterpret_cast<int *>(b->dev[k] + offsetof(BatchHdr, counter)));
     if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return VT_ERR_CUDA;
     if (tp.fp64 && launch_klt_f64(b->dev[k], tp.win, tp.gtype, b->sms * 4, s) != VT_OK) return VT_ERR_CUDA;
     if (ev && ev[3]) cudaEventRecord(ev[3], s);
@@ -301,7 +306,6 @@ vt_status vt_batch_create(int max_frames, int max_tasks, vt_batch **out) {
         ok = ok && cudaMalloc((void **)&b->dev[k], b->tab_bytes) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&b->ev[k], cudaEventDisableTiming) == cudaSuccess;
     }
-    ok = ok && cudaMalloc((void **)&b->counter, 2 * sizeof(int)) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) == cudaSuccess;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -330,7 +334,6 @@ void vt_batch_free(vt_batch *b) {
         if (b->dev[k]) cudaFree(b->dev[k]);
         if (b->ev[k]) cudaEventDestroy(b->ev[k]);
     }
-    if (b->counter) cudaFree(b->counter);
     if (b->cap) cudaStreamDestroy(b->cap);
     free(b);
 }
@@ -403,6 +406,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
     BFrame *bf = reinterpret_cast<BFrame *>(tab + H->off_frames);
     BLvlJob *jobs = reinterpret_cast<BLvlJob *>(tab + H->off_jobs);
     BTileSrc *tsrc = reinterpret_cast<BTileSrc *>(tab + H->off_tsrc);
+    const long tail_limit = nframes <= kTailFewFrames ? kTailFewPx : kTailMaxPx;
     int maxL = 1, maxC = 0;
     for (int f = 0; f < nframes; ++f) {
         const vt_frame_job &fj = frames[f];
@@ -414,7 +418,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
         bf[f].levels = p->levels;
         p->gtype = (int)gtype;
         if (p->levels > maxL) maxL = p->levels;
-        const int c = tail_start_level(p);
+        const int c = tail_start_level(p, tail_limit);
         if (c > maxC) maxC = c;
     }
     for (int l = 0; l < VT_MAX_LEVELS; ++l) {
@@ -422,7 +426,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
         int nj = 0, tiles = 0;
         for (int f = 0; f < nframes; ++f) {
             const vt_pyramid *p = frames[f].pyr;
-            const int c = tail_start_level(p);
+            const int c = tail_start_level(p, tail_limit);
             if (l < VT_MAX_LEVELS - 1) {
                 if (l >= c) continue;  // levels from c on are built by the tail kernel
                 int tx = 0;
@@ -453,7 +457,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
                 // bands per frame capped so that every band of the run gets a
                 // CTA of the tail launch in one round
                 const int cap = b->tail_grid / (nframes > 0 ? nframes : 1);
-                int parts = tail_parts(p);
+                int parts = tail_parts(p, tail_limit);
                 if (parts > cap) parts = cap > 1 ? cap : 1;
                 for (int q = 0; q < parts; ++q) {
                     lj[nj].frame = f;
@@ -500,6 +504,7 @@ vt_status vt_batch_set(vt_batch *b, const vt_frame_job *frames, int nframes, vt_
     tp.klt_grid = klt_grid(b, prm->win, (int)gtype);
     tp.pyr_grid = b->pyr_grid;
     tp.gate = 0;
+    tp.frames = nframes > 0;
     tp.fp64 = H->P.fp64;
     b->staged = k;
     b->next = k ^ 1;
@@ -663,7 +668,7 @@ vt_status vt_batch_info(const vt_batch *b, int *klt_grid_ctas, int *klt_warps_pe
     if (klt_warps_per_cta) *klt_warps_per_cta = b->topo[k].klt_warps;
     if (pyr_grid_ctas) *pyr_grid_ctas = b->topo[k].pyr_grid;
     if (launches_per_run)
-        *launches_per_run = b->staged >= 0 ? b->topo[k].maxL + 1 + 1 + b->topo[k].fp64 + b->topo[k].gate : 0;
+        *launches_per_run = b->staged >= 0 ? b->topo[k].maxL + b->topo[k].frames + 1 + b->topo[k].fp64 + b->topo[k].gate : 0;
     return VT_OK;
 }
 

@@ -160,9 +160,13 @@ struct BLvlJob {
                 // lists tiles_x is the band index and tile0 the band count
 };
 
-// Levels of at most this many pixels are built by the tail kernel, one CTA
-// per frame, entirely in shared memory.
-constexpr int kTailMaxPx = 40960;
+// Levels of at most this many bytes are built by the tail kernel, entirely in
+// shared memory.  One CTA walks a frame's chain of them, so with few frames a
+// level of 24 to 40 KB is better left to one more tiled launch, which all SMs
+// share (one 960x600 frame: 54.5 -> 50.3 us a step, a 1919x1199 build 23.3 ->
+// 20.9); with many frames the chains run side by side and the launch costs
+// more than it gives (32 streams: + 1.7 us).
+constexpr int kTailMaxPx = 40960, kTailFewPx = 24576, kTailFewFrames = 4;
 
 struct BTask {
     const Level *I;  // template pyramid (device level table)
@@ -195,7 +199,8 @@ struct BatchHdr {
     int cap_frames, cap_tasks;
     int off_frames, off_jobs, off_tasks, off_prefix;
     int ngates, gate_points, off_gates, off_gprefix;
-    int off_tsrc, pad_tsrc;  // BTileSrc per tiled job: VT_MAX_LEVELS - 1 lists of cap_frames
+    int off_tsrc;  // BTileSrc per tiled job: VT_MAX_LEVELS - 1 lists of cap_frames
+    int counter;  // the tracking launch's work counter (0 in every staged table)
     vt_gate_params G;
     KParams P;
 };
@@ -209,8 +214,8 @@ bool gate_args_ok(const vt_stereo_rig *rig, const vt_gate_params *prm);
 // `ev` (nullable): one event recorded after each launch (tiled_launches + 1).
 vt_status launch_pyr_batch(const uint8_t *dev_tab, int tiled_launches, int gtype, int grid_pyr, int grid_tail,
                            cudaStream_t s, cudaEvent_t *ev = nullptr);
-int tail_start_level(const vt_pyramid *p);
-int tail_parts(const vt_pyramid *p);
+int tail_start_level(const vt_pyramid *p, long limit);
+int tail_parts(const vt_pyramid *p, long limit);
 int pyr_batch_blocks_per_sm();
 int pyr_tiles(int w, int h, int &tiles_x);
 __host__ __device__ int scharr_tiles(int w, int h, int &tiles_x);

@@ -507,18 +507,18 @@ __host__ __device__ inline bool tail_fits(const Level &L) {
 constexpr int TAIL_SMEM = TAIL_A + TAIL_B;
 
 // First level the tail kernel builds: the first whose rows (at the
-// pyramid's pitch) fit in kTailMaxPx bytes, or the last.
-int tail_start_level(const vt_pyramid *p) {
+// pyramid's pitch) fit in `limit` bytes, or the last.
+int tail_start_level(const vt_pyramid *p, long limit) {
     for (int l = 0; l < p->levels; ++l)
-        if (tail_fits(p->lv[l])) return l;
+        if (tail_fits(p->lv[l]) && (long)p->lv[l].pitch * p->lv[l].h <= limit) return l;
     return p->levels - 1;
 }
 
 // CTAs of a frame's tail: one builds the levels below c, the others (about
 // 4096 pixels each, at most 7) take row bands of level c's gradients.  A last
 // level too large for shared memory is shared tile by tile.
-int tail_parts(const vt_pyramid *p) {
-    const int c = tail_start_level(p);
+int tail_parts(const vt_pyramid *p, long limit) {
+    const int c = tail_start_level(p, limit);
     const long px = (long)p->lv[c].w * p->lv[c].h;
     if (!tail_fits(p->lv[c])) return 8;
     const int n = 1 + (int)((px + 4095) / 4096);
@@ -889,7 +889,7 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
     const Level &L0 = p->lv[0];
     if (img == L0.img && pitch != L0.pitch) return VT_ERR_ARG;
     const bool grad = gtype != VT_GRAD_NONE;
-    const int c = tail_start_level(p);
+    const int c = tail_start_level(p, kTailFewPx);
     const bool small = tail_fits(p->lv[c]);  // the levels from c on take one launch
     // A frame already in level 0 (vt_pyramid_upload) is built in place, and a
     // device image is copied by the launch that reads it first; host images
@@ -937,7 +937,7 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
         e = launch_pdl(!grad                    ? k_pyr_tail_one<VT_GRAD_NONE>
                        : gtype == VT_GRAD_F16 ? k_pyr_tail_one<VT_GRAD_F16>
                                               : k_pyr_tail_one<VT_GRAD_S16>,
-                       grad ? tail_parts(p) : 1, TAIL_THREADS, TAIL_SMEM, s, true, A);
+                       grad ? tail_parts(p, kTailFewPx) : 1, TAIL_THREADS, TAIL_SMEM, s, true, A);
     } else if (e == cudaSuccess && grad) {  // (c is the last level)
         GradJobs gj;
         gj.njobs = 0;
