@@ -291,7 +291,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // below `chunks` of each row.  32 / NCH rows go per step, a lane keeping one
 // chunk of a row: its addresses advance by a constant per step, two
 // instructions per copied chunk (an index split into row and chunk per copy
-// took about 18).
+// took about 18).  Rows that cross the level's first or last one are clamped
+// step by step, unrolled too: half of the windows of the coarse levels do.
 template <int ROWS, int NCH>
 __device__ __forceinline__ void copy_rows(uint32_t dst, const uint8_t *base, int pitch, int y0, int hm1, int chunks,
                                           int lane) {
@@ -307,7 +308,7 @@ __device__ __forceinline__ void copy_rows(uint32_t dst, const uint8_t *base, int
             src += RS * pitch;
         }
     } else {
-#pragma unroll 1
+#pragma unroll
         for (int k = 0; k < STEPS; ++k)
             if (k * RS < rows)
                 cp_async16(d + k * RS * NCH * 16, base + (size_t)clampi(y0 + r + k * RS, 0, hm1) * pitch + 16 * c);
@@ -494,9 +495,10 @@ __device__ __forceinline__ void sample_template(const KCta<WIN> &C, const TWin &
 //   sum r grad T = R - bx Sx - by Sy - bx by Sxy,
 //   R = sum (T - F00) grad T, Sx = sum (F01 - F00) grad T,
 //   Sy = sum (F10 - F00) grad T, Sxy = sum (F11 - F10 - F01 + F00) grad T.
-// The footprint differences are exact (integers); m: R, Sx, Sy, Sxy as (x
-// part, y part).  The footprint is staged
-// in sm.j; w: the level's width.
+// The footprint differences are exact (integers); m: -R, Sx, Sy, Sxy as (x
+// part, y part) -- with R negated, -b is a sum without a sign change, and the
+// negated 1 / det of the step takes it back.  The footprint is staged in sm.j;
+// w: the level's width.
 template <int WIN>
 __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const float (&N)[KRuns<WIN>::NS],
                                              const float2 (&G)[KRuns<WIN>::NS], const KSmem<WIN> &sm,
@@ -521,7 +523,7 @@ __device__ __forceinline__ void cell_moments(int x0, int w, int lane, const floa
             q.y = px_minus(j1[r * JS], q.x);
             if (r > 0) {
                 const int s = i * RL + r - 1;
-                const float e0 = -N[s] - p.x;
+                const float e0 = N[s] + p.x;  // -(T - F00)
                 const float2 d = sub2(q, p);  // F10 - F00, F11 - F10 - F01 + F00
                 a[0] = __ffma2_rn(pair(e0), G[s], a[0]);
                 a[1] = __ffma2_rn(pair(p.y), G[s], a[1]);
@@ -962,7 +964,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         // eta = G^-1 b in grey/px units: G = unit^2 G_s, b = unit b_s => eta = adj(G_s) b_s / (unit det_s)
         // (unit is a power of two, so det * unit is exact; the adjugate
         // products cancel for ill-conditioned G, hence kdiff)
-        const float inv_det = 1.0f / (det * unit) * kImgUnscale;  // b carries the image scale
+        const float inv_det = -1.0f / (det * unit) * kImgUnscale;  // of -b, which carries the image scale
         if (!inside) {
             o.status = 0;
             o.reason = VT_LOST_OOB;
@@ -986,9 +988,9 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
         bool left_cell = false;  // whether sm.cell_* hold this level's entries
         for (int k = 1;; ++k) {
             const float bxy = bx * by;
-            float2 b = __ffma2_rn(pair(-bx), m[1], m[0]);
-            b = __ffma2_rn(pair(-by), m[2], b);
-            b = __ffma2_rn(pair(-bxy), m[3], b);
+            float2 b = __ffma2_rn(pair(bx), m[1], m[0]);  // -b
+            b = __ffma2_rn(pair(by), m[2], b);
+            b = __ffma2_rn(pair(bxy), m[3], b);
             const float ex = kdiff(g22, b.x, g12, b.y) * inv_det;
             const float ey = kdiff(g11, b.y, g12, b.x) * inv_det;
             nux += ex;
