@@ -12,6 +12,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import re
+import sys
 from dataclasses import dataclass
 
 from . import build as _build
@@ -95,10 +96,12 @@ def header_functions() -> list:
 def _ptr(x):
     if x is None:
         return None
+    try:
+        return x.data_ptr()
+    except AttributeError:
+        pass
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if hasattr(x, "ctypes"):
         return x.ctypes.data
     raise TypeError(f"cannot take the address of {type(x)}")
@@ -106,9 +109,13 @@ def _ptr(x):
 
 def _stream(s):
     if s is None:
-        import torch
+        torch = sys.modules.get("torch")
+        if torch is None or not torch.cuda.is_initialized():
+            import torch
 
-        return torch.cuda.current_stream().cuda_stream
+            return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle without a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(s, int):
         return s
     return s.cuda_stream
@@ -599,6 +606,24 @@ _sig("vt_stereo_gate", i32, [vp, vp, vp, i32, C.POINTER(vt_stereo_rig), C.POINTE
 VT_LOST_DISP, VT_LOST_DEPTH, VT_LOST_REPROJ = 5, 6, 7
 
 
+_DOUBLES = {n: C.c_double * n for n in (3, 4, 9)}
+
+
+def _doubles(v, n):
+    """n doubles of a flat tuple or list of numbers, or of anything numpy flattens to n values."""
+    if type(v) in (tuple, list) and len(v) == n:
+        try:
+            return _DOUBLES[n](*v)
+        except TypeError:  # nested, or not plain numbers
+            pass
+    import numpy as np
+
+    a = np.ascontiguousarray(v, np.float64)
+    if a.size != n:
+        raise ValueError(f"expected {n} values, got {a.size}")
+    return _DOUBLES[n].from_buffer_copy(a)
+
+
 @dataclass
 class StereoRig:
     """Pinhole intrinsics (fx, fy, cx, cy) of both cameras and the left-to-right
@@ -609,15 +634,7 @@ class StereoRig:
     t: tuple = (0.0, 0.0, 0.0)
 
     def c(self) -> vt_stereo_rig:
-        import numpy as np
-
-        def flat(v, n):
-            a = np.asarray(v, np.float64).ravel()
-            if a.size != n:
-                raise ValueError(f"expected {n} values, got {a.size}")
-            return (C.c_double * n)(*a.tolist())
-
-        return vt_stereo_rig(flat(self.kl, 4), flat(self.kr, 4), flat(self.R, 9), flat(self.t, 3))
+        return vt_stereo_rig(_doubles(self.kl, 4), _doubles(self.kr, 4), _doubles(self.R, 9), _doubles(self.t, 3))
 
 
 @dataclass
