@@ -789,10 +789,10 @@ static void add_grad_job(GradJobs &jobs, int &blocks, const Level &lv, const uin
 // (programmatic dependent launch): a build is a chain of launches of a few
 // microseconds each, and the launch latency between them cost as much as the
 // kernels.
-static vt_status launch_scharr(const GradJobs &jobs, int total_blocks, int gtype, cudaStream_t s) {
+static vt_status launch_scharr(const GradJobs &jobs, int total_blocks, int gtype, bool pdl, cudaStream_t s) {
     if (jobs.njobs == 0 || total_blocks == 0) return VT_OK;
     return launch_pdl(gtype == VT_GRAD_F16 ? k_scharr<VT_GRAD_F16> : k_scharr<VT_GRAD_S16>, total_blocks, SC_THREADS, 0,
-                      s, true, jobs) == cudaSuccess
+                      s, pdl, jobs) == cudaSuccess
                ? VT_OK
                : VT_ERR_CUDA;
 }
@@ -860,19 +860,29 @@ static vt_status check_build_args(const uint8_t *img, int w, int h, int pitch, i
     return VT_OK;
 }
 
-// Whether a kernel on the current device may read `p` as it is: its own
-// memory, managed or pinned host memory (anything else is left to the copy
-// call, which reaches other devices and refuses what it cannot read).
-static bool kernel_readable(const void *p) {
+// Where a kernel on the current device can read the image at `p`: its own or
+// managed memory, or pinned host memory (*host is then set); null for anything
+// else, which is left to the copy call (it reaches other devices and pageable
+// memory, and refuses what it cannot read).
+static const uint8_t *kernel_readable(const uint8_t *p, bool *host) {
     cudaPointerAttributes a;
     int dev = 0;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return nullptr;
     }
-    return a.type == cudaMemoryTypeManaged || a.type == cudaMemoryTypeHost ||
-           (a.type == cudaMemoryTypeDevice && a.device == dev);
+    *host = a.type == cudaMemoryTypeHost;
+    if (*host || a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev))
+        return static_cast<const uint8_t *>(a.devicePointer);
+    return nullptr;
 }
+
+// Pinned host frames up to this size, and larger ones whose rows need a new
+// pitch, are read by the first launch over the host link: a 2-D copy moves
+// rows at a third of the link's rate and costs a launch of its own (752 x 480:
+// 41 -> 16 us a build, 1437 x 901: 66 -> 28).  A large frame in one piece is
+// copied faster than a kernel reads it (1920 x 1200 alone: 47 against 51 us).
+constexpr size_t kHostReadBytes = (size_t)1 << 20;
 
 static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int levels, int img_on_device, int gtype,
                             void *cuda_stream, vt_pyramid **out) {
@@ -892,9 +902,15 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
     const int c = tail_start_level(p, kTailFewPx);
     const bool small = tail_fits(p->lv[c]);  // the levels from c on take one launch
     // A frame already in level 0 (vt_pyramid_upload) is built in place, and a
-    // device image is copied by the launch that reads it first; host images
-    // (and one-level pyramids without planes) are copied up first.
-    const bool by_kernel = img_on_device && img != L0.img && (c > 0 || small || grad) && kernel_readable(img);
+    // device image is copied by the launch that reads it first; other host
+    // images (and one-level pyramids without planes) are copied up first.
+    bool from_host = false, by_kernel = false;
+    if (img != L0.img && (c > 0 || small || grad) &&
+        (img_on_device || pitch != L0.pitch || (size_t)pitch * h <= kHostReadBytes)) {
+        const uint8_t *q = kernel_readable(img, &from_host);
+        by_kernel = q != nullptr;
+        if (by_kernel) img = q;
+    }
     cudaError_t e = cudaSuccess;
     if (img != L0.img && !by_kernel) {
         e = cudaMemcpy2DAsync(L0.img, L0.pitch, img, pitch, w, h,
@@ -921,7 +937,7 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
         e = launch_pdl(!grad                    ? k_pyrdown<false, VT_GRAD_S16>
                        : gtype == VT_GRAD_F16 ? k_pyrdown<true, VT_GRAD_F16>
                                               : k_pyrdown<true, VT_GRAD_S16>,
-                       tiles, PD_THREADS, 0, s, true, j);
+                       tiles, PD_THREADS, 0, s, l > 0 || !from_host, j);  // (host memory: after the launch before)
     }
     if (e == cudaSuccess && small) {
         static const bool attr = tail_smem_ok(k_pyr_tail_one<VT_GRAD_S16>) && tail_smem_ok(k_pyr_tail_one<VT_GRAD_F16>) &&
@@ -937,14 +953,14 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
         e = launch_pdl(!grad                    ? k_pyr_tail_one<VT_GRAD_NONE>
                        : gtype == VT_GRAD_F16 ? k_pyr_tail_one<VT_GRAD_F16>
                                               : k_pyr_tail_one<VT_GRAD_S16>,
-                       grad ? tail_parts(p, kTailFewPx) : 1, TAIL_THREADS, TAIL_SMEM, s, true, A);
+                       grad ? tail_parts(p, kTailFewPx) : 1, TAIL_THREADS, TAIL_SMEM, s, c > 0 || !from_host, A);
     } else if (e == cudaSuccess && grad) {  // (c is the last level)
         GradJobs gj;
         gj.njobs = 0;
         int blocks = 0;
         add_grad_job(gj, blocks, p->lv[c], c == 0 ? img : p->lv[c].img, c == 0 ? pitch : p->lv[c].pitch,
                      c == 0 ? vec_ok : 1);
-        if (launch_scharr(gj, blocks, gtype, s) != VT_OK) e = cudaErrorLaunchFailure;
+        if (launch_scharr(gj, blocks, gtype, c > 0 || !from_host, s) != VT_OK) e = cudaErrorLaunchFailure;
     }
     if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         cudaGetLastError();
@@ -981,7 +997,7 @@ vt_status vt_gradients(vt_pyramid *p, vt_grad_type t, void *cuda_stream) {
     gj.njobs = 0;
     int blocks = 0;
     for (int l = 0; l < p->levels; ++l) add_grad_job(gj, blocks, p->lv[l], p->lv[l].img, p->lv[l].pitch, 1);
-    const vt_status st = launch_scharr(gj, blocks, (int)t, (cudaStream_t)cuda_stream);
+    const vt_status st = launch_scharr(gj, blocks, (int)t, true, (cudaStream_t)cuda_stream);
     if (st == VT_OK) p->gtype = (int)t;
     return st;
 }

@@ -50,3 +50,33 @@ def test_every_width(h, grad):
                     ex = np.stack([ref.gx[l], ref.gy[l]], -1).astype(np.float32) / 32
                     assert np.array_equal(g.view(np.uint16), ex.astype(np.float16).view(np.uint16)), (img.shape, l)
     b.free()
+
+
+@pytest.mark.parametrize("grad", [1, 0])
+def test_pinned_host_images(grad):
+    """Pinned host frames, read by the first launch (small ones, and rows that
+    need a new pitch) or copied up (a large frame in one piece), rewritten on
+    the host between builds; and a pageable one."""
+    import torch
+
+    import paper_2607_01757_gb300 as vt
+
+    rng = np.random.Generator(np.random.PCG64(grad))
+    for w, h, L in [(1, 1, 1), (63, 40, 2), (128, 96, 1), (641, 479, 4), (704, 300, 3), (1280, 1024, 3), (1283, 900, 2)]:
+        pin = torch.empty((h, w), dtype=torch.uint8, pin_memory=True)
+        p = vt.vt_pyramid_create(w, h, L)
+        for k in range(3):
+            img = rng.integers(0, 256, (h, w), dtype=np.uint8)
+            src = pin if k < 2 else torch.from_numpy(img)
+            src.copy_(torch.from_numpy(img))
+            if grad:
+                vt.vt_pyramid_build_grad(src, L, vt.VT_GRAD_S16, out=p)
+            else:
+                vt.vt_pyramid_build(src, L, out=p)
+            torch.cuda.synchronize()
+            ref = oracle.build_pyramid(img, L)
+            for l in range(L):
+                assert np.array_equal(p.level(l).cpu().numpy(), ref.levels[l]), (w, h, k, l)
+                if grad:
+                    g = p.grad(l).cpu().numpy()
+                    assert np.array_equal(g[..., 0], ref.gx[l]) and np.array_equal(g[..., 1], ref.gy[l]), (w, h, k, l)
