@@ -13,6 +13,8 @@
 // The same staged tile serves the pyramid step and, in the fused variant, the
 // gradients of the source level and the copy of a caller's frame.  A frame's
 // small levels are built together from shared memory (tail_build).
+#include <cuda.h>
+
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -860,21 +862,37 @@ static vt_status check_build_args(const uint8_t *img, int w, int h, int pitch, i
     return VT_OK;
 }
 
-// Where a kernel on the current device can read the image at `p`: its own or
-// managed memory, or pinned host memory (*host is then set); null for anything
-// else, which is left to the copy call (it reaches other devices and pageable
-// memory, and refuses what it cannot read).
-static const uint8_t *kernel_readable(const uint8_t *p, bool *host) {
-    cudaPointerAttributes a;
-    int dev = 0;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+// Where a kernel on the current device can read the `bytes` bytes at `p`: in
+// the device's own memory (on_device) or in pinned host memory (not
+// on_device), wholly inside one allocation; null for anything else, which is
+// left to the copy call (it reaches other devices and pageable memory, and
+// refuses what it cannot read).
+static const uint8_t *kernel_readable(const uint8_t *p, size_t bytes, bool on_device) {
+    typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = []() -> Query {  // once, thread-safe static initialisation
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) ==
+                            cudaSuccess &&
+                        r == cudaDriverEntryPointSuccess;
+        if (!ok) cudaGetLastError();
+        return ok ? reinterpret_cast<Query>(f) : nullptr;
+    }();
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0;
+    int of = -1, dev = -2;
+    CUdeviceptr at = 0, start = 0;
+    size_t size = 0;
+    void *to[] = {&type, &of, &at, &start, &size};
+    if (!query || cudaGetDevice(&dev) != cudaSuccess || query(5, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) {
         cudaGetLastError();
         return nullptr;
     }
-    *host = a.type == cudaMemoryTypeHost;
-    if (*host || a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev))
-        return static_cast<const uint8_t *>(a.devicePointer);
-    return nullptr;
+    const bool ok = (on_device ? type == CU_MEMORYTYPE_DEVICE && of == dev : type == CU_MEMORYTYPE_HOST) && at >= start &&
+                    at - start <= size && bytes <= size - (at - start);
+    return ok ? reinterpret_cast<const uint8_t *>((uintptr_t)at) : nullptr;
 }
 
 // Pinned host frames up to this size, and larger ones whose rows need a new
@@ -904,13 +922,14 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
     // A frame already in level 0 (vt_pyramid_upload) is built in place, and a
     // device image is copied by the launch that reads it first; other host
     // images (and one-level pyramids without planes) are copied up first.
-    bool from_host = false, by_kernel = false;
+    bool by_kernel = false;
     if (img != L0.img && (c > 0 || small || grad) &&
         (img_on_device || pitch != L0.pitch || (size_t)pitch * h <= kHostReadBytes)) {
-        const uint8_t *q = kernel_readable(img, &from_host);
+        const uint8_t *q = kernel_readable(img, (size_t)pitch * (h - 1) + w, img_on_device != 0);
         by_kernel = q != nullptr;
         if (by_kernel) img = q;
     }
+    const bool from_host = by_kernel && !img_on_device;
     cudaError_t e = cudaSuccess;
     if (img != L0.img && !by_kernel) {
         e = cudaMemcpy2DAsync(L0.img, L0.pitch, img, pitch, w, h,
