@@ -69,3 +69,14 @@ def test_selection_over_many_chunks(min_dist):
                         block_radius=1, border=2)
     _same([noise, dots], prm)
     _same([synth.make_config1(2).I] * 8 + [noise], vt.GfttParams(max_corners=300, min_dist=min_dist))
+
+
+@pytest.mark.parametrize("min_dist", [46340, 65536])
+def test_min_dist_wider_than_any_level(min_dist):
+    """A distance whose square passes 32 bits: the best corner alone is kept,
+    also of more candidates than a chunk holds."""
+    import paper_2607_01757_gb300 as vt
+
+    rng = np.random.Generator(np.random.PCG64(5))
+    prm = vt.GfttParams(max_corners=500, quality=0.0, min_dist=min_dist, nms_radius=3, block_radius=1, border=2)
+    _same([rng.integers(0, 256, (480, 752), dtype=np.uint8)], prm)
