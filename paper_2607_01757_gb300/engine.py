@@ -233,11 +233,20 @@ class BatchedTracker:
             vt.vt_pyramid_build_grad(img, levels, self.grad_type, stream, out=out)
 
     def plain_launches(self, sids, n_t, n_s, gate=True):
-        """Kernel launches of plain_step (the level-0 copy is a memcpy, not a kernel)."""
+        """Kernel launches of plain_step.  A build takes one launch a level down
+        to the first of at most 24,576 bytes (rows at a pitch of 64), and one
+        for the levels from there on (without planes only if the last level
+        needs no more than 40,960)."""
         n = 0
         for k, i in enumerate(sids):
             s = self.streams[i]
-            per_pyr = (s.levels - 1) + (0 if self.grad_type == vt.VT_GRAD_NONE else 1)
+            sizes = []
+            w, h = s.w, s.h
+            for _ in range(s.levels):
+                sizes.append((w + 63) // 64 * 64 * h)
+                w, h = (w + 1) // 2, (h + 1) // 2
+            c = next((l for l, b in enumerate(sizes) if b <= 24576), s.levels - 1)
+            per_pyr = c + int(self.grad_type != vt.VT_GRAD_NONE or sizes[c] <= 40960)
             n += per_pyr * (2 if s.stereo else 1)
             n += int(n_t[k] > 0) + int(s.stereo and n_s[k] > 0)
             n += int(s.stereo and n_s[k] > 0 and s.rig is not None and gate)
