@@ -6,11 +6,13 @@
 //
 //   k_tracks_carry  survivors of the temporal step (status 1) in index order,
 //                   ages + 1, sorted by (age desc, index asc) in shared
-//                   memory; the greedy min-distance thinning in that order is
-//                   resolved in parallel rounds over a cell grid in shared
-//                   memory (a survivor is kept when no kept higher-priority
-//                   survivor lies closer than min_dist, dropped when one
-//                   does); kept survivors rewrite the pool in priority order
+//                   memory (a pool these kernels wrote is in that order and
+//                   only checked); the greedy min-distance thinning in that
+//                   order finds each survivor's closer higher-priority ones
+//                   over a cell grid in shared memory and resolves them in
+//                   parallel rounds (a survivor is kept when no kept
+//                   higher-priority survivor lies closer than min_dist,
+//                   dropped when one does); kept survivors rewrite the pool in priority order
 //                   and, optionally, a detector mask padded with NaN.
 //   k_tracks_spawn  accepted detections, in their priority order, appended
 //                   until the pool holds `cap` features, with identities
@@ -24,9 +26,10 @@
 
 namespace vt {
 
-constexpr int TK_THREADS = 1024;
-constexpr int TK_PER = VT_POOL_MAX / TK_THREADS;  // pool entries per thread
-constexpr int TK_MAX_CELLS = 4096;
+constexpr int TK_THREADS = 1024;    // threads of the largest CTA
+constexpr int TK_MAX_CELLS = 8192;  // the grid's cells: at most TK_CELLS_PER a
+constexpr int TK_MIN_CELLS = 4096;  // survivor, within these limits
+constexpr int TK_CELLS_PER = 8;
 constexpr int kMaxPoolJobs = 192;
 enum : uint8_t { TK_UNDECIDED = 0, TK_KEPT = 1, TK_DROPPED = 2 };
 
@@ -41,8 +44,7 @@ struct SpawnJobs {
     vt_spawn_job j[kMaxPoolJobs];
 };
 
-// Exclusive block-wide scan of one int per thread (TK_THREADS threads);
-// returns the total through *total.
+// Exclusive block-wide scan of one int per thread; the total through *total.
 __device__ __forceinline__ int block_scan(int v, int *warp_sums, int *total) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int x = v;
@@ -53,20 +55,16 @@ __device__ __forceinline__ int block_scan(int v, int *warp_sums, int *total) {
     }
     if (lane == 31) warp_sums[wid] = x;
     __syncthreads();
-    if (wid == 0) {
-        int s = warp_sums[lane];
+    int s = lane < (int)(blockDim.x >> 5) ? warp_sums[lane] : 0;  // every warp sums the warps for itself
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        warp_sums[lane] = s;  // inclusive sums of the warps
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
     }
-    __syncthreads();
-    const int excl = x - v + (wid > 0 ? warp_sums[wid - 1] : 0);
-    if (total) *total = warp_sums[31];
-    __syncthreads();
-    return excl;
+    *total = __shfl_sync(0xffffffffu, s, 31);
+    const int before = __shfl_sync(0xffffffffu, s, wid > 0 ? wid - 1 : 0);
+    __syncthreads();  // warp_sums may be written again
+    return x - v + (wid > 0 ? before : 0);
 }
 
 __device__ __forceinline__ float dist2(float2 a, float2 b) {
@@ -75,39 +73,62 @@ __device__ __forceinline__ float dist2(float2 a, float2 b) {
 }
 
 struct CarrySmem {
-    unsigned long long key[VT_POOL_MAX];  // (age << 32) | ~rank, sorted descending
-    float2 pos[VT_POOL_MAX];              // survivor positions by survivor rank
+    float2 pos[VT_POOL_MAX];               // survivor positions by survivor rank
+    float2 sorted[VT_POOL_MAX];            // and by priority, where that is another order
     int32_t id[VT_POOL_MAX];
-    int32_t age[VT_POOL_MAX];  // already + 1
-    int16_t cell_of[VT_POOL_MAX];          // by priority position
-    int16_t member[VT_POOL_MAX];           // priority positions grouped by cell
-    int cell_start[TK_MAX_CELLS + 1];
-    int cursor[TK_MAX_CELLS];
-    uint8_t state[VT_POOL_MAX];            // by priority position
+    int32_t age[VT_POOL_MAX];              // already + 1
+    union {
+        unsigned long long key[VT_POOL_MAX];  // (age << 32) | ~rank, sorted descending
+        short4 closer[VT_POOL_MAX];           // by priority: the first closer higher-priority survivors (see k_tracks_carry)
+    };
+    int16_t rank[VT_POOL_MAX];             // of the survivor at a priority position
+    int16_t next[VT_POOL_MAX];             // a cell's survivors, linked from its head
+    int head[TK_MAX_CELLS];
+    uint8_t state[VT_POOL_MAX];
     int warp_sums[32];
     float red[4][32];
 };
 
-__global__ void __launch_bounds__(TK_THREADS) k_tracks_carry(const __grid_constant__ CarryJobs J) {
+// Calls f(o) for the survivors o of higher priority than q that lie closer to
+// it than min_dist, until f returns false.
+template <typename F>
+__device__ __forceinline__ void each_closer(const CarrySmem &S, const float2 *pos, int q, int ix, int iy, int cx, int cy,
+                                            float md2, F &&f) {
+    const float2 p = pos[q];
+    for (int yy = max(0, iy - 1); yy <= min(cy - 1, iy + 1); ++yy)
+        for (int xx = max(0, ix - 1); xx <= min(cx - 1, ix + 1); ++xx)
+            for (int o = S.head[yy * cx + xx]; o >= 0; o = S.next[o])
+                if (o < q && dist2(p, pos[o]) < md2 && !f(o)) return;
+}
+
+// Bound by latency: one CTA per pool, dependent reads and barriers.  A pool as
+// the last carry-over and spawning left it needs no sort (66 passes over the
+// keys of 2,000 survivors), and the grid is walked once: a survivor's first
+// three closer ones of higher priority are kept in `closer`, so a round reads
+// three states.  Cold caches, launch included: 8 pools of 250 25 -> 12.5 us,
+// 32 of 1,000 41 -> 18, 32 of 2,000 67 -> 22; out of order, 32 of 1,000
+// 39 -> 29.  Most of what is left is the launch and three dependent reads from
+// memory (count, status, positions).
+__global__ void __launch_bounds__(TK_THREADS, 1) k_tracks_carry(const __grid_constant__ CarryJobs J) {
     extern __shared__ __align__(16) uint8_t tk_smem[];
     CarrySmem &S = *reinterpret_cast<CarrySmem *>(tk_smem);
     const vt_carry_job &jb = J.j[blockIdx.x];
     const vt_track_pool &P = jb.pool;
-    const int n = min(*P.count, P.cap);
     const float2 *tracked = reinterpret_cast<const float2 *>(jb.tracked);
-    const int t = threadIdx.x;
-    // 1. survivors in index order (TK_PER consecutive entries per thread)
+    const int t = threadIdx.x, T = blockDim.x;
+    pdl_wait();  // the tracked positions may be the previous kernel's output
+    const int n = min(*P.count, P.cap);
+    // 1. survivors in index order (`per` consecutive entries per thread)
+    const int per = (n + T - 1) / T;
     int mine = 0;
-#pragma unroll
-    for (int k = 0; k < TK_PER; ++k) {
-        const int i = t * TK_PER + k;
+    for (int k = 0; k < per; ++k) {
+        const int i = t * per + k;
         mine += (i < n && jb.status[i] != 0) ? 1 : 0;
     }
     int m;
     int r = block_scan(mine, S.warp_sums, &m);
-#pragma unroll
-    for (int k = 0; k < TK_PER; ++k) {
-        const int i = t * TK_PER + k;
+    for (int k = 0; k < per; ++k) {
+        const int i = t * per + k;
         if (i < n && jb.status[i] != 0) {
             S.pos[r] = tracked[i];
             S.id[r] = P.ids[i];
@@ -116,31 +137,44 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_carry(const __grid_consta
         }
     }
     __syncthreads();
-    // 2. priority order: age descending, then survivor rank ascending (bitonic, descending keys)
-    int N = 1;
-    while (N < m) N <<= 1;
-    for (int i = t; i < N; i += TK_THREADS)
-        S.key[i] = i < m ? ((unsigned long long)(uint32_t)S.age[i] << 32) | (0xffffffffu - (unsigned)i) : 0ull;
-    __syncthreads();
-    for (int k = 2; k <= N; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = t; i < N; i += TK_THREADS) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const unsigned long long a = S.key[i], b = S.key[p];
-                    if (((i & k) == 0) ? (a < b) : (a > b)) {
-                        S.key[i] = b;
-                        S.key[p] = a;
+    // 2. priority order: age descending, then survivor rank ascending
+    int unsorted = 0;
+    for (int i = t; i + 1 < m; i += T) unsorted |= (uint32_t)S.age[i] < (uint32_t)S.age[i + 1];
+    const float2 *pos = S.pos;  // by priority
+    if (__syncthreads_or(unsorted)) {
+        int N = 1;
+        while (N < m) N <<= 1;
+        for (int i = t; i < N; i += T)
+            S.key[i] = i < m ? ((unsigned long long)(uint32_t)S.age[i] << 32) | (0xffffffffu - (unsigned)i) : 0ull;
+        __syncthreads();
+        for (int k = 2; k <= N; k <<= 1)  // bitonic, descending keys
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int i = t; i < N; i += T) {
+                    const int p = i ^ j;
+                    if (p > i) {
+                        const unsigned long long a = S.key[i], b = S.key[p];
+                        if (((i & k) == 0) ? (a < b) : (a > b)) {
+                            S.key[i] = b;
+                            S.key[p] = a;
+                        }
                     }
                 }
+                __syncthreads();
             }
-            __syncthreads();
+        for (int q = t; q < m; q += T) {
+            const int s = 0xffffffffu - (unsigned)(S.key[q] & 0xffffffffu);
+            S.rank[q] = (int16_t)s;
+            S.sorted[q] = S.pos[s];
         }
+        pos = S.sorted;
+    } else {
+        for (int q = t; q < m; q += T) S.rank[q] = (int16_t)q;
+    }
     // 3. cell grid over the survivors' bounding box: cells wider than
     //    min_dist (by 0.1 %, so rounding cannot separate a close pair by two
-    //    cells), at most TK_MAX_CELLS of them
+    //    cells); a cell holds less than a survivor of a spread-out pool
     float lo_x = INFINITY, lo_y = INFINITY, hi_x = -INFINITY, hi_y = -INFINITY;
-    for (int i = t; i < m; i += TK_THREADS) {
+    for (int i = t; i < m; i += T) {
         const float2 p = S.pos[i];
         if (!isfinite(p.x) || !isfinite(p.y)) continue;  // non-finite points share cell 0
         lo_x = fminf(lo_x, p.x);
@@ -162,21 +196,26 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_carry(const __grid_consta
         S.red[3][t >> 5] = hi_y;
     }
     __syncthreads();
-    lo_x = S.red[0][0], lo_y = S.red[1][0], hi_x = S.red[2][0], hi_y = S.red[3][0];
-    for (int w = 1; w < 32; ++w) {
-        lo_x = fminf(lo_x, S.red[0][w]);
-        lo_y = fminf(lo_y, S.red[1][w]);
-        hi_x = fmaxf(hi_x, S.red[2][w]);
-        hi_y = fmaxf(hi_y, S.red[3][w]);
+    {  // (every warp reduces the warps' boxes for itself)
+        const int w = min(t & 31, (T >> 5) - 1);
+        lo_x = S.red[0][w], lo_y = S.red[1][w], hi_x = S.red[2][w], hi_y = S.red[3][w];
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        lo_x = fminf(lo_x, __shfl_xor_sync(0xffffffffu, lo_x, o));
+        lo_y = fminf(lo_y, __shfl_xor_sync(0xffffffffu, lo_y, o));
+        hi_x = fmaxf(hi_x, __shfl_xor_sync(0xffffffffu, hi_x, o));
+        hi_y = fmaxf(hi_y, __shfl_xor_sync(0xffffffffu, hi_y, o));
     }
     const float md = J.min_dist, md2 = __fmul_rn(md, md);
     float cs = md * 1.001f;
     int cx = 1, cy = 1;
     if (lo_x <= hi_x && lo_y <= hi_y) {  // some finite survivor
+        const float most = (float)min(TK_MAX_CELLS, max(TK_MIN_CELLS, TK_CELLS_PER * m));
         int tries = 0;
         for (;; ++tries) {
             const float fx = floorf((hi_x - lo_x) / cs) + 1.f, fy = floorf((hi_y - lo_y) / cs) + 1.f;
-            if (fx * fy <= (float)TK_MAX_CELLS) {
+            if (fx * fy <= most) {
                 cx = (int)fx;
                 cy = (int)fy;
                 break;
@@ -187,90 +226,77 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_carry(const __grid_consta
     } else {
         lo_x = lo_y = 0.f;
     }
-    for (int c = t; c < TK_MAX_CELLS; c += TK_THREADS) S.cursor[c] = 0;
+    for (int c = t; c < cx * cy; c += T) S.head[c] = -1;
     __syncthreads();
-    for (int q = t; q < m; q += TK_THREADS) {  // q: priority position
-        const float2 p = S.pos[0xffffffffu - (unsigned)(S.key[q] & 0xffffffffu)];
-        const int ix = clampi((int)floorf((p.x - lo_x) / cs), 0, cx - 1);
-        const int iy = clampi((int)floorf((p.y - lo_y) / cs), 0, cy - 1);
-        const int c = ix + cx * iy;
-        S.cell_of[q] = (int16_t)c;
-        atomicAdd(&S.cursor[c], 1);
-        S.state[q] = TK_UNDECIDED;
+    auto cell = [&](float2 p, int &ix, int &iy) {
+        ix = clampi((int)floorf((p.x - lo_x) / cs), 0, cx - 1);
+        iy = clampi((int)floorf((p.y - lo_y) / cs), 0, cy - 1);
+    };
+    for (int q = t; q < m; q += T) {  // q: priority position
+        int ix, iy;
+        cell(pos[q], ix, iy);
+        S.next[q] = (int16_t)atomicExch(&S.head[iy * cx + ix], q);
     }
     __syncthreads();
-    {  // cell starts: exclusive scan of the counts (TK_MAX_CELLS / TK_THREADS cells per thread)
-        constexpr int CPT = TK_MAX_CELLS / TK_THREADS;
-        int cnt[CPT], sum = 0;
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            cnt[k] = S.cursor[t * CPT + k];
-            sum += cnt[k];
-        }
-        int run = block_scan(sum, S.warp_sums, nullptr);
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            S.cell_start[t * CPT + k] = run;
-            S.cursor[t * CPT + k] = run;
-            run += cnt[k];
-        }
-        if (t == TK_THREADS - 1) S.cell_start[TK_MAX_CELLS] = run;
+    // 4. greedy thinning.  Each survivor's closer ones of higher priority: the
+    //    first three, and w = -2 if there are more; with none it is kept.
+    for (int q = t; q < m; q += T) {
+        int ix, iy, found = 0;
+        cell(pos[q], ix, iy);
+        short4 c = make_short4(-1, -1, -1, -1);
+        each_closer(S, pos, q, ix, iy, cx, cy, md2, [&](int o) {
+            if (found == 0) c.x = (short)o;
+            else if (found == 1) c.y = (short)o;
+            else if (found == 2) c.z = (short)o;
+            else c.w = -2;
+            return ++found < 4;
+        });
+        S.closer[q] = c;
+        S.state[q] = found ? TK_UNDECIDED : TK_KEPT;
     }
     __syncthreads();
-    // members of each cell (order within a cell does not matter)
-    for (int q = t; q < m; q += TK_THREADS) S.member[atomicAdd(&S.cursor[S.cell_of[q]], 1)] = (int16_t)q;
-    __syncthreads();
-    // 4. greedy thinning in parallel rounds
+    //    Rounds: the undecided survivor of highest priority is decided in each.
     for (;;) {
         int undecided = 0;
-        for (int q = t; q < m; q += TK_THREADS) {
-            if (S.state[q] != TK_UNDECIDED) continue;
-            const float2 p = S.pos[0xffffffffu - (unsigned)(S.key[q] & 0xffffffffu)];
-            const int c = S.cell_of[q], ccx = c % cx, ccy = c / cx;
-            bool blocked = false, dropped = false;
-            for (int dy = -1; dy <= 1 && !dropped; ++dy) {
-                const int yy = ccy + dy;
-                if (yy < 0 || yy >= cy) continue;
-                for (int dx = -1; dx <= 1 && !dropped; ++dx) {
-                    const int xx = ccx + dx;
-                    if (xx < 0 || xx >= cx) continue;
-                    const int cc = yy * cx + xx;
-                    for (int e = S.cell_start[cc]; e < S.cell_start[cc + 1]; ++e) {
-                        const int o = S.member[e];
-                        if (o >= q) continue;  // lower priority (or itself)
-                        const float2 po = S.pos[0xffffffffu - (unsigned)(S.key[o] & 0xffffffffu)];
-                        if (!(dist2(p, po) < md2)) continue;
-                        const uint8_t so = *reinterpret_cast<volatile uint8_t *>(&S.state[o]);
-                        if (so == TK_KEPT) {
-                            dropped = true;
-                            break;
-                        }
-                        if (so == TK_UNDECIDED) blocked = true;
-                    }
-                }
+        for (int q = t; q < m; q += T) {
+            volatile uint8_t *state = S.state;
+            if (state[q] != TK_UNDECIDED) continue;
+            const short4 c = S.closer[q];
+            const uint8_t sx = state[c.x], sy = c.y >= 0 ? state[c.y] : (uint8_t)TK_DROPPED,
+                          sz = c.z >= 0 ? state[c.z] : (uint8_t)TK_DROPPED;
+            bool dropped = sx == TK_KEPT || sy == TK_KEPT || sz == TK_KEPT;
+            bool blocked = sx == TK_UNDECIDED || sy == TK_UNDECIDED || sz == TK_UNDECIDED;
+            if (c.w == -2 && !dropped && !blocked) {  // the three are dropped: all of them
+                int ix, iy;
+                cell(pos[q], ix, iy);
+                each_closer(S, pos, q, ix, iy, cx, cy, md2, [&](int o) {
+                    const uint8_t so = state[o];
+                    dropped = so == TK_KEPT;
+                    blocked |= so == TK_UNDECIDED;
+                    return !dropped;
+                });
             }
-            if (dropped) S.state[q] = TK_DROPPED;
-            else if (!blocked) S.state[q] = TK_KEPT;
+            if (dropped) state[q] = TK_DROPPED;
+            else if (!blocked) state[q] = TK_KEPT;
             else undecided = 1;
         }
         if (!__syncthreads_or(undecided)) break;
     }
     // 5. the kept survivors, in priority order, rewrite the pool
+    const int perm = (m + T - 1) / T;
     int kept_mine = 0;
-#pragma unroll
-    for (int k = 0; k < TK_PER; ++k) {
-        const int q = t * TK_PER + k;
+    for (int k = 0; k < perm; ++k) {
+        const int q = t * perm + k;
         kept_mine += (q < m && S.state[q] == TK_KEPT) ? 1 : 0;
     }
     int kept;
     int w = block_scan(kept_mine, S.warp_sums, &kept);
     float2 *pts = reinterpret_cast<float2 *>(P.pts);
     float2 *mask = reinterpret_cast<float2 *>(jb.mask);
-#pragma unroll
-    for (int k = 0; k < TK_PER; ++k) {
-        const int q = t * TK_PER + k;
+    for (int k = 0; k < perm; ++k) {
+        const int q = t * perm + k;
         if (q < m && S.state[q] == TK_KEPT) {
-            const int s = 0xffffffffu - (unsigned)(S.key[q] & 0xffffffffu);
+            const int s = S.rank[q];
             pts[w] = S.pos[s];
             P.ids[w] = S.id[s];
             P.ages[w] = S.age[s];
@@ -279,7 +305,7 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_carry(const __grid_consta
         }
     }
     if (mask)
-        for (int i = kept + t; i < P.cap; i += TK_THREADS) mask[i] = make_float2(NAN, NAN);
+        for (int i = kept + t; i < P.cap; i += T) mask[i] = make_float2(NAN, NAN);
     if (t == 0) *P.count = kept;
 }
 
@@ -287,12 +313,14 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_spawn(const __grid_consta
     __shared__ int warp_sums[32];
     const vt_spawn_job &jb = J.j[blockIdx.x];
     const vt_track_pool &P = jb.pool;
+    const int T = blockDim.x;
+    pdl_wait();  // the detections may be the previous kernel's output
     const int c0 = min(*P.count, P.cap), nc = *jb.n_corners;
     const int room = P.cap - c0, id0 = *P.next_id;
     const float2 *corners = reinterpret_cast<const float2 *>(jb.corners);
     float2 *pts = reinterpret_cast<float2 *>(P.pts);
     int base = 0;
-    for (int b0 = 0; b0 < nc && base < room; b0 += TK_THREADS) {  // chunks of TK_THREADS detections, in order
+    for (int b0 = 0; b0 < nc && base < room; b0 += T) {  // chunks of T detections, in order
         const int i = b0 + threadIdx.x;
         const int a = (i < nc && (!jb.accept || jb.accept[i] != 0)) ? 1 : 0;
         int total;
@@ -310,6 +338,16 @@ __global__ void __launch_bounds__(TK_THREADS) k_tracks_spawn(const __grid_consta
         *P.count = c0 + added;
         *P.next_id = id0 + added;
     }
+}
+
+// Threads of a call's CTAs: an entry of the largest pool each, where that fits
+// (8 pools of 250: 12.3 us with 256 threads, 12.9 with 512, 15.0 with 1,024).
+template <typename Job>
+static int pool_threads(const Job *jobs, int njobs) {
+    int cap = 128;
+    for (int i = 0; i < njobs; ++i)
+        if (jobs[i].pool.cap > cap) cap = jobs[i].pool.cap;
+    return cap >= TK_THREADS ? TK_THREADS : (cap + 31) / 32 * 32;
 }
 
 static bool pool_ok(const vt_track_pool &p) {
@@ -337,8 +375,9 @@ vt_status vt_tracks_carry(const vt_carry_job *jobs, int njobs, float min_dist, v
                                     (int)sizeof(CarrySmem)) == cudaSuccess;
     }();
     (void)attr;
-    k_tracks_carry<<<njobs, TK_THREADS, sizeof(CarrySmem), (cudaStream_t)cuda_stream>>>(J);
-    return cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
+    const cudaError_t e = launch_pdl(k_tracks_carry, njobs, pool_threads(jobs, njobs), sizeof(CarrySmem),
+                                     (cudaStream_t)cuda_stream, true, J);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
 }
 
 vt_status vt_tracks_spawn(const vt_spawn_job *jobs, int njobs, void *cuda_stream) {
@@ -349,8 +388,9 @@ vt_status vt_tracks_spawn(const vt_spawn_job *jobs, int njobs, void *cuda_stream
     SpawnJobs J;
     J.n = njobs;
     for (int i = 0; i < njobs; ++i) J.j[i] = jobs[i];
-    k_tracks_spawn<<<njobs, TK_THREADS, 0, (cudaStream_t)cuda_stream>>>(J);
-    return cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
+    const cudaError_t e =
+        launch_pdl(k_tracks_spawn, njobs, pool_threads(jobs, njobs), 0, (cudaStream_t)cuda_stream, true, J);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
 }
 
 }  // extern "C"
