@@ -45,9 +45,9 @@ SM_MAX_MHZ = 2070.0
 # for that workload and only while the sources still hash the same: a kernel
 # changed since the capture reports null.
 NCU_CAPTURES = {
-    "k_klt_batch": {"bytes": 438424320 + 4009728, "date": "2026-12-04", "sources_sha1": "20c723f569bf5e384dbcff33684c4ae7f4b04791"},
-    "pyramid": {"bytes": 63668480 + 203302912 + 15835392 + 11063296 + 3412480 + 0 + 1634304 + 0,
-                "date": "2026-12-04", "sources_sha1": "e5833bb23c3f9284e8d5b2711cfce13ba8f93983"},
+    "k_klt_batch": {"bytes": 438413824 + 4111616, "date": "2026-12-05", "sources_sha1": "5ffb96676637c02d83524822be030ee8aad58992"},
+    "pyramid": {"bytes": 62096384 + 202794752 + 15792896 + 10516736 + 3411968 + 0 + 1636864 + 256,
+                "date": "2026-12-05", "sources_sha1": "94e8dcaab148ac73bd521a8c2898dfe46e047f14"},
 }
 # the pyramid launches' tiles and tail bands are laid out by the batch's host code
 KERNEL_SOURCES = {

@@ -190,8 +190,8 @@ __device__ __forceinline__ GateOut gate_point(const GateArgs &g, float2 pl, floa
 // spectrum has no gap, or when any decision lies within 1e-8 (relative) of its
 // threshold -- a million times the rounding of either route -- so both take
 // the same decisions.  Not-a-numbers fail these tests and go there, too.
-// Measured: 19,000 pairs 77 -> 13 us, about 6,000 pairs of a batched run 77 ->
-// 14 us (one warp a CTA spreads them; cold caches); no pair of either is left
+// Measured: 19,000 pairs 78 -> 11.4 us, about 6,000 pairs of a batched run 76 ->
+// 14.7 us (one warp a CTA spreads them; cold caches); no pair of either is left
 // to gate_point.
 
 // One FP32 Jacobi rotation in the (P, Q) plane (see jacobi_rotate).
