@@ -379,7 +379,7 @@ int orc_gftt(const int16_t *gx, const int16_t *gy, int w, int h, int gpitch, int
                 const volatile float dx = (float)x - (float)mask[2 * m];
                 const volatile float dy = (float)y - (float)mask[2 * m + 1];
                 const volatile float dd = dx * dx + dy * dy;
-                if (dd < (float)(min_dist * min_dist)) ok = 0;
+                if (dd < (float)((long)min_dist * min_dist)) ok = 0;
             }
             if (!ok) continue;
             if (n == cap) {
