@@ -115,11 +115,7 @@ __global__ void __launch_bounds__(128) k_klt_batch_f64(const uint8_t *tab) {
 template <int WIN, int GT>
 static void launch_f64_win(const uint8_t *tab, int grid, cudaStream_t s) {
     const size_t smem = KCta<WIN>::bytes(4);
-    static const bool attr = [smem] {  // once, thread-safe static initialisation
-        return cudaFuncSetAttribute(k_klt_batch_f64<WIN, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem) == cudaSuccess;
-    }();
-    (void)attr;
+    smem_opt_in<k_klt_batch_f64<WIN, GT>>(smem);  // (refused: so is the launch)
     k_klt_batch_f64<WIN, GT><<<grid, 128, smem, s>>>(tab);
 }
 
@@ -155,12 +151,7 @@ struct KltBatchKernel {
 template <int WIN, int GT, int WARPS>
 static KltBatchKernel klt_batch_entry() {
     const size_t smem = KCta<WIN>::bytes(WARPS);
-    // opt in to more than 48 KB where needed (once, thread-safe static initialisation)
-    static const bool attr = [smem] {
-        return cudaFuncSetAttribute(k_klt_batch<WIN, GT, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem) == cudaSuccess;
-    }();
-    (void)attr;
+    smem_opt_in<k_klt_batch<WIN, GT, WARPS>>(smem);  // (refused: so is the launch)
     return {k_klt_batch<WIN, GT, WARPS>, smem};
 }
 

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "vt.h"
 
 namespace vt {
@@ -77,6 +79,25 @@ inline cudaError_t launch_pdl(void (*k)(Params...), int grid, int block, size_t 
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+// Allow launches of `Kernel` with `bytes` (the same on every call) of dynamic
+// shared memory on the current device.  The allowance belongs to a device, so
+// it is asked for once on each.
+template <auto Kernel>
+inline bool smem_opt_in(size_t bytes) {
+    constexpr int kDevices = 64;
+    static std::atomic<bool> done[kDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        if (dev < kDevices && done[dev].load(std::memory_order_acquire)) return true;
+        if (cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) {
+            if (dev < kDevices) done[dev].store(true, std::memory_order_release);
+            return true;
+        }
+    }
+    cudaGetLastError();
+    return false;
 }
 
 // ---------------------------------------------------------------- pyramid jobs

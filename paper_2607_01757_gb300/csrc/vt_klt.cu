@@ -68,28 +68,21 @@ __global__ void k_fb_check(const float2 *p0, const float2 *p1, const uint8_t *sf
 }
 
 template <int WIN, int GT, bool FB, bool F64>
-static void launch_pass(const KltArgs &A, cudaStream_t s) {
+static bool launch_pass(const KltArgs &A, cudaStream_t s) {
     const int blocks = (A.n + KLT_WARPS - 1) / KLT_WARPS;
     const size_t smem = KCta<WIN>::bytes(KLT_WARPS);
-    if (smem > 48 * 1024) {
-        static const bool attr = [smem] {  // once, thread-safe static initialisation
-            return cudaFuncSetAttribute(k_klt<WIN, GT, FB, F64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem) == cudaSuccess;
-        }();
-        (void)attr;
-    }
+    if (smem > 48 * 1024 && !smem_opt_in<k_klt<WIN, GT, FB, F64>>(smem)) return false;
     // launched while the stream's previous kernel ends (programmatic dependent
     // launch): the tables are filled meanwhile
-    launch_pdl(k_klt<WIN, GT, FB, F64>, blocks, KLT_WARPS * 32, smem, s, true, A);
+    return launch_pdl(k_klt<WIN, GT, FB, F64>, blocks, KLT_WARPS * 32, smem, s, true, A) == cudaSuccess;
 }
 
 // The FP32 launch, then (only when an accepted template can be
 // ill-conditioned, fp64_needed) the FP64-capable launch over its pending points.
 template <int WIN, int GT, bool FB>
 static vt_status launch_one(const KltArgs &A, cudaStream_t s) {
-    launch_pass<WIN, GT, FB, false>(A, s);
-    if (A.P.fp64) launch_pass<WIN, GT, FB, true>(A, s);
-    return cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
+    const bool ok = launch_pass<WIN, GT, FB, false>(A, s) && (!A.P.fp64 || launch_pass<WIN, GT, FB, true>(A, s));
+    return cudaGetLastError() == cudaSuccess && ok ? VT_OK : VT_ERR_CUDA;
 }
 
 template <int GT, bool FB>

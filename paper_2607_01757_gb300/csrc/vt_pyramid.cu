@@ -737,16 +737,12 @@ __host__ __device__ int scharr_tiles(int w, int h, int &tiles_x) {
     return tiles_x * ((h + SC_TH - 1) / SC_TH);
 }
 
-template <typename K>
-static bool tail_smem_ok(K *k) {
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_SMEM) == cudaSuccess;
-}
-
 vt_status launch_pyr_batch(const uint8_t *dev_tab, int tiled_launches, int gtype, int grid_pyr, int grid_tail,
                            cudaStream_t s, cudaEvent_t *ev) {
-    static const bool attr = tail_smem_ok(k_pyr_tail<VT_GRAD_S16>) && tail_smem_ok(k_pyr_tail<VT_GRAD_F16>) &&
-                             tail_smem_ok(k_pyr_tail<VT_GRAD_NONE>);  // once, thread-safe static initialisation
-    (void)attr;
+    if (!(gtype == VT_GRAD_F16    ? smem_opt_in<k_pyr_tail<VT_GRAD_F16>>(TAIL_SMEM)
+          : gtype == VT_GRAD_NONE ? smem_opt_in<k_pyr_tail<VT_GRAD_NONE>>(TAIL_SMEM)
+                                  : smem_opt_in<k_pyr_tail<VT_GRAD_S16>>(TAIL_SMEM)))
+        return VT_ERR_CUDA;
     // every launch after the first overlaps its start with the previous one's
     // end (programmatic dependent launch), except where an event is recorded
     // in between for per-launch timing
@@ -959,9 +955,6 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
                        tiles, PD_THREADS, 0, s, l > 0 || !from_host, j);  // (host memory: after the launch before)
     }
     if (e == cudaSuccess && small) {
-        static const bool attr = tail_smem_ok(k_pyr_tail_one<VT_GRAD_S16>) && tail_smem_ok(k_pyr_tail_one<VT_GRAD_F16>) &&
-                                 tail_smem_ok(k_pyr_tail_one<VT_GRAD_NONE>);  // once, thread-safe static initialisation
-        (void)attr;
         TailArgs A;
         for (int l = 0; l < VT_MAX_LEVELS; ++l) A.lv[l] = l < levels ? p->lv[l] : Level{};
         A.levels = levels;
@@ -969,10 +962,14 @@ static vt_status build_impl(const uint8_t *img, int w, int h, int pitch, int lev
         A.img = img;
         A.pitch = pitch;
         A.vec_ok = vec_ok;
-        e = launch_pdl(!grad                    ? k_pyr_tail_one<VT_GRAD_NONE>
-                       : gtype == VT_GRAD_F16 ? k_pyr_tail_one<VT_GRAD_F16>
-                                              : k_pyr_tail_one<VT_GRAD_S16>,
-                       grad ? tail_parts(p, kTailFewPx) : 1, TAIL_THREADS, TAIL_SMEM, s, c > 0 || !from_host, A);
+        const bool fits = !grad                    ? smem_opt_in<k_pyr_tail_one<VT_GRAD_NONE>>(TAIL_SMEM)
+                          : gtype == VT_GRAD_F16 ? smem_opt_in<k_pyr_tail_one<VT_GRAD_F16>>(TAIL_SMEM)
+                                                 : smem_opt_in<k_pyr_tail_one<VT_GRAD_S16>>(TAIL_SMEM);
+        e = !fits ? cudaErrorInvalidValue
+                  : launch_pdl(!grad                    ? k_pyr_tail_one<VT_GRAD_NONE>
+                               : gtype == VT_GRAD_F16 ? k_pyr_tail_one<VT_GRAD_F16>
+                                                      : k_pyr_tail_one<VT_GRAD_S16>,
+                               grad ? tail_parts(p, kTailFewPx) : 1, TAIL_THREADS, TAIL_SMEM, s, c > 0 || !from_host, A);
     } else if (e == cudaSuccess && grad) {  // (c is the last level)
         GradJobs gj;
         gj.njobs = 0;

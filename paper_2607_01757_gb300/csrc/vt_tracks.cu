@@ -370,11 +370,7 @@ vt_status vt_tracks_carry(const vt_carry_job *jobs, int njobs, float min_dist, v
     J.n = njobs;
     J.min_dist = min_dist;
     for (int i = 0; i < njobs; ++i) J.j[i] = jobs[i];
-    static const bool attr = [] {  // once, thread-safe static initialisation
-        return cudaFuncSetAttribute(k_tracks_carry, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(CarrySmem)) == cudaSuccess;
-    }();
-    (void)attr;
+    if (!smem_opt_in<k_tracks_carry>(sizeof(CarrySmem))) return VT_ERR_CUDA;
     const cudaError_t e = launch_pdl(k_tracks_carry, njobs, pool_threads(jobs, njobs), sizeof(CarrySmem),
                                      (cudaStream_t)cuda_stream, true, J);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? VT_OK : VT_ERR_CUDA;
