@@ -57,15 +57,14 @@ __device__ __forceinline__ void scharr_at(const uint8_t (*s)[IW], int sr, int sc
     dy = 3 * (a20 - a00) + 10 * (a21 - a01) + 3 * (a22 - a02);
 }
 
-// 16 bytes at any address, by the aligned words that hold them (each holds at
-// least one of the bytes, so none lies outside the caller's allocation).
-__device__ __forceinline__ uint4 load16_any(const uint8_t *p) {
+// `n` bytes (1 .. 16) at any address, by the aligned words that hold them (each
+// holds at least one of the bytes, so none lies outside the caller's allocation).
+__device__ __forceinline__ uint4 load16_any(const uint8_t *p, unsigned n) {
     const unsigned a = (unsigned)(uintptr_t)p & 3u;
     const uint32_t *q = reinterpret_cast<const uint32_t *>(p - a);
     uint32_t v[5];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = __ldg(q + k);
-    v[4] = a ? __ldg(q + 4) : 0u;
+    for (int k = 0; k < 5; ++k) v[k] = 4 * k < a + n ? q[k] : 0u;
     return make_uint4(__funnelshift_r(v[0], v[1], 8 * a), __funnelshift_r(v[1], v[2], 8 * a),
                       __funnelshift_r(v[2], v[3], 8 * a), __funnelshift_r(v[3], v[4], 8 * a));
 }
@@ -73,28 +72,42 @@ __device__ __forceinline__ uint4 load16_any(const uint8_t *p) {
 // Stage rows [iy0, iy0 + IH) and columns [ix0, ix0 + IW) of an image (ix0 a
 // multiple of 16), rows and columns reflected into it; ends with a barrier.
 // The 16-byte chunks inside the image are copied whole (one load where the
-// rows are 16-byte aligned, vec_ok, else word by word), the chunk that holds the last column byte by byte (a caller's
-// last row may end there); the columns -2, -1, w and w + 1 are then filled
+// rows are 16-byte aligned, vec_ok, else word by word), of the chunk that holds
+// the last column only the words that reach into the row (a caller's last row
+// may end there); the columns -2, -1, w and w + 1 are then filled
 // from the staged ones (the reflected columns lie in the same tile for w >= 4;
 // the readers use no others outside the image).  A tile at the image's edge
 // so costs about what an inner one does: mapping every byte of it through the
 // reflection took most of a small level's launch (all of its tiles are at an
 // edge): 11.7 -> 4.5 us at 752 x 480, and level 0 of 32 frames 144 -> 89 us.
+//
+// Pixels are read by ordinary loads, here and in tail_build: the launch before
+// may still be writing them when this one starts (programmatic dependent
+// launch), and a read-only load (__ldg) wants data that nothing writes while
+// the kernel runs; it need not stay behind pdl_wait() either.  A thread's
+// chunks are all loaded before the first is stored, which the compiler does not
+// do for ordinary loads by itself (752 x 480 build 13.44 us without, 12.38 so;
+// 12.94 with read-only loads; 1919 x 1199 half planes 21.0, 17.8 and 20.7).
 template <int IH, int IW>
 __device__ __forceinline__ void stage_tile(uint8_t (*s)[IW], const uint8_t *src, int w, int h, int pitch, int ix0,
                                            int iy0, bool vec_ok) {
     constexpr int C16 = IW / 16;
     if (w >= 4) {
         const bool inner = ix0 >= 0 && ix0 + IW <= w && iy0 >= 0 && iy0 + IH <= h;
-        for (int i = threadIdx.x; i < IH * C16; i += blockDim.x) {
-            const int r = i / C16, c = i - r * C16, x = ix0 + 16 * c;
-            const uint8_t *row = src + (size_t)(inner ? iy0 + r : refl101(iy0 + r, h)) * pitch;
-            if (inner || (x >= 0 && x + 16 <= w)) {
-                *reinterpret_cast<uint4 *>(&s[r][c * 16]) =
-                    vec_ok ? __ldg(reinterpret_cast<const uint4 *>(row + x)) : load16_any(row + x);
-            } else if (x >= 0 && x < w) {
-                for (int q = 0; x + q < w; ++q) s[r][c * 16 + q] = __ldg(row + x + q);
+        constexpr int N = (IH * C16 + PD_THREADS - 1) / PD_THREADS;  // chunks a thread (of at least PD_THREADS)
+        uint4 v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int i = threadIdx.x + k * blockDim.x, r = i / C16, x = ix0 + 16 * (i - r * C16);
+            if (i < IH * C16 && (inner || (x >= 0 && x < w))) {
+                const uint8_t *p = src + (size_t)(inner ? iy0 + r : refl101(iy0 + r, h)) * pitch + x;
+                v[k] = vec_ok && x + 16 <= w ? *reinterpret_cast<const uint4 *>(p) : load16_any(p, min(16, w - x));
             }
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int i = threadIdx.x + k * blockDim.x, r = i / C16, c = i - r * C16, x = ix0 + 16 * c;
+            if (i < IH * C16 && (inner || (x >= 0 && x < w))) *reinterpret_cast<uint4 *>(&s[r][c * 16]) = v[k];
         }
         if (!inner) {
             __syncthreads();
@@ -114,7 +127,7 @@ __device__ __forceinline__ void stage_tile(uint8_t (*s)[IW], const uint8_t *src,
         for (int i = threadIdx.x; i < IH * IW; i += blockDim.x) {
             const int r = i / IW, c = i - r * IW;
             const int sy = refl101(iy0 + r, h), sx = refl101(ix0 + c, w);
-            s[r][c] = __ldg(src + (size_t)sy * pitch + sx);
+            s[r][c] = src[(size_t)sy * pitch + sx];
         }
     }
     __syncthreads();
@@ -639,7 +652,7 @@ __device__ __forceinline__ void tail_build(const Level *lv, int levels, int c, i
             const int C = (w + 15) / 16;
             for (int i = threadIdx.x; i < (r1 - r0) * C; i += blockDim.x) {
                 const int y = r0 + i / C, k = i % C;
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(Lc.img + (size_t)y * Lc.pitch) + k);
+                const uint4 v = reinterpret_cast<const uint4 *>(Lc.img + (size_t)y * Lc.pitch)[k];
                 uint32_t *d = reinterpret_cast<uint32_t *>(cur + y * S) + 1 + 4 * k;
                 const int room = S / 4 - 1 - 4 * k;  // words left in the row
                 if (room > 0) d[0] = v.x;
