@@ -23,6 +23,9 @@ struct KltArgs {
     KParams P;
 };
 
+static_assert(alignof(KltArgs) % 16 == 0 && offsetof(KltArgs, I) % 16 == 0 && offsetof(KltArgs, J) % 16 == 0,
+              "level tables are copied in 16-byte pieces");
+
 // F64 = false: the FP32 tracker; a point with an ill-conditioned level is
 // left pending (status kStatusPending).  F64 = true: the second launch,
 // which tracks only the pending points, with such levels in FP64.

@@ -36,7 +36,8 @@
 
 namespace vt {
 
-struct KPyr {
+// (aligned for the 16-byte loads of track_point_dir, as a kernel parameter too)
+struct __align__(16) KPyr {
     Level lv[VT_MAX_LEVELS];
 };
 
@@ -175,7 +176,7 @@ __device__ __forceinline__ float pow2neg(int l) { return __int_as_float((127 - l
 // level's template is copied in while this level iterates) -- in win + 1 rows
 // of NC (image) or NG (gradients) 16-byte chunks.
 template <int WIN>
-struct KSmem {
+struct __align__(16) KSmem {
     static constexpr int NC = (WIN + 31) / 16;  // 16-byte chunks per staged row: cover 15 + win + 1 bytes
     static constexpr int JS = NC * 16;          // staged row stride in bytes
     static_assert(JS >= 15 + WIN + 1, "a staged row covers the footprint row");
@@ -1085,6 +1086,7 @@ __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, 
     // the two level tables next to the warp: a level's fields are one shared
     // load away, not a chain of global ones
     static_assert(sizeof(Level) * VT_MAX_LEVELS == 16 * 16, "16 lanes copy a table");
+    static_assert(offsetof(KSmem<WIN>, lv) % 16 == 0 && alignof(KSmem<WIN>) >= 16, "16-byte stores");
     __syncwarp();
     reinterpret_cast<uint4 *>(sm.lv)[lane] = reinterpret_cast<const uint4 *>(lane < 16 ? I : J)[lane & 15];
     __syncwarp();
