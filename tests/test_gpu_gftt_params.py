@@ -1,5 +1,6 @@
-"""Minimum distances whose square passes 32 bits, and levels wide enough for
-squared distances that do: masks and selection, compared for equality."""
+"""The ends of the detector's parameters -- minimum distances whose square passes
+32 bits, levels wide enough for squared distances that do, qualities from zero
+to infinity --: masks and selection, compared for equality."""
 
 import numpy as np
 import pytest
@@ -36,3 +37,13 @@ def test_wide_level(min_dist):
     prm = vt.GfttParams(max_corners=40, quality=0.3, min_dist=min_dist, nms_radius=4, border=1)
     _same([_frame(65535, 12, 3)], prm)
     _same([_frame(12, 65535, 4)], prm, [np.array([[6.0, 2000.0]], np.float32)])
+
+
+@pytest.mark.parametrize("quality", [0.0, -0.0, 1e-45, 1.0, 1.5, float("inf")])
+@pytest.mark.parametrize("nms", [2, 4])
+def test_quality_at_its_ends(quality, nms):
+    """Both zeros admit every local maximum, 1 the frame's best, more none."""
+    import paper_2607_01757_gb300 as vt
+
+    prm = vt.GfttParams(max_corners=300, quality=quality, min_dist=5, nms_radius=nms)
+    _same([_frame(320, 200, 1), np.full((60, 80), 9, np.uint8)], prm)
