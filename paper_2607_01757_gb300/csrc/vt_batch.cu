@@ -576,13 +576,13 @@ vt_status vt_batch_run_timed(vt_batch *b, void *cuda_stream, void *ev_pyr0, void
 vt_status vt_batch_run_levels_timed(vt_batch *b, void *cuda_stream, void **events, int nevents) {
     if (!b || b->staged < 0 || !events || nevents < 0) return VT_ERR_ARG;
     const int k = b->staged;
-    const int need = b->topo[k].maxL + 1 + 4;
+    const int need = 4 + b->topo[k].maxL + b->topo[k].frames;  // (no pyramid launch without frames)
     if (nevents < need) return VT_ERR_ARG;
     b->fresh = false;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     cudaEvent_t ev[4] = {(cudaEvent_t)events[0], (cudaEvent_t)events[1], (cudaEvent_t)events[2],
                          (cudaEvent_t)events[3]};
-    vt_status st = enqueue(b, k, s, ev, reinterpret_cast<cudaEvent_t *>(events + 4));
+    vt_status st = enqueue(b, k, s, ev, nevents > 4 ? reinterpret_cast<cudaEvent_t *>(events + 4) : nullptr);
     if (st != VT_OK) return st;
     if (cudaEventRecord(b->ev[k], s) != cudaSuccess) {
         cudaGetLastError();
