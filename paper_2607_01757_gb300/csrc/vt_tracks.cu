@@ -12,7 +12,8 @@
 //                   over a cell grid in shared memory and resolves them in
 //                   parallel rounds (a survivor is kept when no kept
 //                   higher-priority survivor lies closer than min_dist,
-//                   dropped when one does); kept survivors rewrite the pool in priority order
+//                   dropped when one does), or one by one where they crowd
+//                   (greedy_in_order); kept survivors rewrite the pool in priority order
 //                   and, optionally, a detector mask padded with NaN.
 //   k_tracks_spawn  accepted detections, in their priority order, appended
 //                   until the pool holds `cap` features, with identities
@@ -22,6 +23,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "vt_greedy.cuh"
 #include "vt_internal.cuh"
 
 namespace vt {
@@ -31,7 +33,11 @@ constexpr int TK_MAX_CELLS = 8192;  // the grid's cells: at most TK_CELLS_PER a
 constexpr int TK_MIN_CELLS = 4096;  // survivor, within these limits
 constexpr int TK_CELLS_PER = 8;
 constexpr int kMaxPoolJobs = 192;
-enum : uint8_t { TK_UNDECIDED = 0, TK_KEPT = 1, TK_DROPPED = 2 };
+// Pools left to greedy_in_order: where a survivor would have to look at more than
+// TK_WALK others (TK_WALK_LARGE in pools of more than TK_THREADS, where it costs
+// up to 128 steps of 7 us), or TK_ROUNDS rounds have not settled the pool.
+constexpr int TK_WALK = 32, TK_WALK_LARGE = 128, TK_ROUNDS = 8;
+enum : uint8_t { TK_UNDECIDED = GR_UNDECIDED, TK_KEPT = GR_KEPT, TK_DROPPED = GR_DROPPED };
 
 struct CarryJobs {
     int n;
@@ -87,18 +93,23 @@ struct CarrySmem {
     uint8_t state[VT_POOL_MAX];
     int warp_sums[32];
     float red[4][32];
+    GreedySmem greedy;
 };
 
 // Calls f(o) for the survivors o of higher priority than q that lie closer to
-// it than min_dist, until f returns false.
+// it than min_dist, until f returns false; false when more than `left`
+// survivors would have to be looked at.
 template <typename F>
-__device__ __forceinline__ void each_closer(const CarrySmem &S, const float2 *pos, int q, int ix, int iy, int cx, int cy,
-                                            float md2, F &&f) {
+__device__ __forceinline__ bool each_closer(const CarrySmem &S, const float2 *pos, int q, int ix, int iy, int cx, int cy,
+                                            float md2, int left, F &&f) {
     const float2 p = pos[q];
     for (int yy = max(0, iy - 1); yy <= min(cy - 1, iy + 1); ++yy)
         for (int xx = max(0, ix - 1); xx <= min(cx - 1, ix + 1); ++xx)
-            for (int o = S.head[yy * cx + xx]; o >= 0; o = S.next[o])
-                if (o < q && dist2(p, pos[o]) < md2 && !f(o)) return;
+            for (int o = S.head[yy * cx + xx]; o >= 0; o = S.next[o]) {
+                if (left-- == 0) return false;
+                if (o < q && dist2(p, pos[o]) < md2 && !f(o)) return true;
+            }
+    return true;
 }
 
 // Bound by latency: one CTA per pool, dependent reads and barriers.  A pool as
@@ -108,7 +119,11 @@ __device__ __forceinline__ void each_closer(const CarrySmem &S, const float2 *po
 // three states.  Cold caches, launch included: 8 pools of 250 25 -> 12.5 us,
 // 32 of 1,000 41 -> 18, 32 of 2,000 67 -> 22; out of order, 32 of 1,000
 // 39 -> 29.  Most of what is left is the launch and three dependent reads from
-// memory (count, status, positions).
+// memory (count, status, positions).  Crowded pools are left to greedy_in_order
+// (one pool, launches of its set-up included): 60 / 1,000 / 4,096 survivors in one
+// place 25 / 31 / 59 us (in rounds 235 / 449 / 43,000), a line of 4,096 each in
+// conflict with the two before it 738 (2,170), 4,096 spread over 10 min_dist
+// squared 89 (1,640).
 __global__ void __launch_bounds__(TK_THREADS, 1) k_tracks_carry(const __grid_constant__ CarryJobs J) {
     extern __shared__ __align__(16) uint8_t tk_smem[];
     CarrySmem &S = *reinterpret_cast<CarrySmem *>(tk_smem);
@@ -240,23 +255,26 @@ __global__ void __launch_bounds__(TK_THREADS, 1) k_tracks_carry(const __grid_con
     __syncthreads();
     // 4. greedy thinning.  Each survivor's closer ones of higher priority: the
     //    first three, and w = -2 if there are more; with none it is kept.
+    const int walk = m <= TK_THREADS ? TK_WALK : TK_WALK_LARGE;
+    int crowded = 0;
     for (int q = t; q < m; q += T) {
         int ix, iy, found = 0;
         cell(pos[q], ix, iy);
         short4 c = make_short4(-1, -1, -1, -1);
-        each_closer(S, pos, q, ix, iy, cx, cy, md2, [&](int o) {
+        const bool all = each_closer(S, pos, q, ix, iy, cx, cy, md2, walk, [&](int o) {
             if (found == 0) c.x = (short)o;
             else if (found == 1) c.y = (short)o;
             else if (found == 2) c.z = (short)o;
             else c.w = -2;
             return ++found < 4;
         });
+        crowded |= !all;
         S.closer[q] = c;
         S.state[q] = found ? TK_UNDECIDED : TK_KEPT;
     }
-    __syncthreads();
+    crowded = __syncthreads_or(crowded);
     //    Rounds: the undecided survivor of highest priority is decided in each.
-    for (;;) {
+    for (int round = 0; !crowded; ++round) {
         int undecided = 0;
         for (int q = t; q < m; q += T) {
             volatile uint8_t *state = S.state;
@@ -269,18 +287,25 @@ __global__ void __launch_bounds__(TK_THREADS, 1) k_tracks_carry(const __grid_con
             if (c.w == -2 && !dropped && !blocked) {  // the three are dropped: all of them
                 int ix, iy;
                 cell(pos[q], ix, iy);
-                each_closer(S, pos, q, ix, iy, cx, cy, md2, [&](int o) {
+                const bool all = each_closer(S, pos, q, ix, iy, cx, cy, md2, walk, [&](int o) {
                     const uint8_t so = state[o];
                     dropped = so == TK_KEPT;
                     blocked |= so == TK_UNDECIDED;
                     return !dropped;
                 });
+                blocked |= !all;
             }
             if (dropped) state[q] = TK_DROPPED;
             else if (!blocked) state[q] = TK_KEPT;
             else undecided = 1;
         }
         if (!__syncthreads_or(undecided)) break;
+        crowded = round + 1 == TK_ROUNDS;
+    }
+    if (crowded) {  // the same decisions one by one
+        for (int q = t; q < m; q += T) S.state[q] = TK_UNDECIDED;
+        __syncthreads();
+        greedy_in_order(S.state, m, S.greedy, [&](int a, int b) { return dist2(pos[a], pos[b]) < md2; });
     }
     // 5. the kept survivors, in priority order, rewrite the pool
     const int perm = (m + T - 1) / T;
