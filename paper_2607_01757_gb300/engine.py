@@ -235,8 +235,9 @@ class BatchedTracker:
     def plain_launches(self, sids, n_t, n_s, gate=True):
         """Kernel launches of plain_step.  A build takes one launch a level down
         to the first of at most 24,576 bytes (rows at a pitch of 64), and one
-        for the levels from there on (without planes only if the last level
-        needs no more than 40,960)."""
+        for the levels from there on (without planes only if that leaves
+        something to do: levels below it, or the frame's copy, and no more than
+        40,960 bytes; vt_pyramid.cu, build_impl)."""
         n = 0
         for k, i in enumerate(sids):
             s = self.streams[i]
@@ -246,7 +247,7 @@ class BatchedTracker:
                 sizes.append((w + 63) // 64 * 64 * h)
                 w, h = (w + 1) // 2, (h + 1) // 2
             c = next((l for l, b in enumerate(sizes) if b <= 24576), s.levels - 1)
-            per_pyr = c + int(self.grad_type != vt.VT_GRAD_NONE or sizes[c] <= 40960)
+            per_pyr = c + int(self.grad_type != vt.VT_GRAD_NONE or (sizes[c] <= 40960 and (c == 0 or c + 1 < s.levels)))
             n += per_pyr * (2 if s.stereo else 1)
             n += int(n_t[k] > 0) + int(s.stereo and n_s[k] > 0)
             n += int(s.stereo and n_s[k] > 0 and s.rig is not None and gate)

@@ -3,13 +3,14 @@
  * the real runtime refuses it, when it wants more dynamic shared memory than
  * the kernel has been allowed on the current device.  Linked with the
  * library's own objects in place of the runtime. */
+#include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <stdlib.h>
 #include <string.h>
 
 #define API __attribute__((visibility("default")))
 
-static int device, launches, refused;
+static int device, launches, refused, copies;
 static cudaError_t last;
 static struct { const void *f; int dev, bytes; } allowed[1024];
 static int n_allowed;
@@ -17,6 +18,25 @@ static int n_allowed;
 API void fake_set_device(int d) { device = d; }
 API int fake_launches(void) { return launches; }
 API int fake_refused(void) { return refused; }
+API int fake_copies(void) { return copies; }
+
+/* The one range of pinned host memory, for the pointer query. */
+static CUdeviceptr pinned;
+static size_t pinned_bytes;
+API void fake_pin(void *p, size_t n) { pinned = (CUdeviceptr)p; pinned_bytes = n; }
+static CUresult query(unsigned n, CUpointer_attribute *what, void **to, CUdeviceptr p)
+{
+    if (p < pinned || p >= pinned + pinned_bytes) return CUDA_ERROR_INVALID_VALUE;
+    for (unsigned i = 0; i < n; ++i) switch (what[i]) {
+        case CU_POINTER_ATTRIBUTE_MEMORY_TYPE: *(unsigned *)to[i] = CU_MEMORYTYPE_HOST; break;
+        case CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL: *(int *)to[i] = 0; break;
+        case CU_POINTER_ATTRIBUTE_DEVICE_POINTER: *(CUdeviceptr *)to[i] = p; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_START_ADDR: *(CUdeviceptr *)to[i] = pinned; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_SIZE: *(size_t *)to[i] = pinned_bytes; break;
+        default: return CUDA_ERROR_INVALID_VALUE;
+    }
+    return CUDA_SUCCESS;
+}
 
 static cudaError_t err(cudaError_t e) { if (e) last = e; return e; }
 
@@ -96,6 +116,7 @@ cudaError_t cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size
                               cudaStream_t st)
 {
     (void)k; (void)st;
+    ++copies;
     for (size_t y = 0; y < h; ++y) memcpy((char *)d + y * dp, (const char *)s + y * sp, w);
     return cudaSuccess;
 }
@@ -104,9 +125,11 @@ cudaError_t cudaGetSymbolAddress(void **p, const void *s) { *p = (void *)s; retu
 cudaError_t cudaGetDriverEntryPointByVersion(const char *n, void **f, unsigned v, unsigned long long fl,
                                              enum cudaDriverEntryPointQueryResult *r)
 {
-    (void)n; (void)v; (void)fl; (void)r;
-    *f = NULL;
-    return err(cudaErrorNotSupported);
+    (void)v; (void)fl;
+    if (strcmp(n, "cuPointerGetAttributes")) return err(cudaErrorNotSupported);
+    *f = (void *)query;
+    *r = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *f, int b, size_t s)
 {
