@@ -648,27 +648,24 @@ __device__ __forceinline__ void tail_build(const Level *lv, int levels, int c, i
         if (!chain && (GT == VT_GRAD_NONE || y0 >= y1)) return;
         const int r0 = chain ? 0 : max(0, y0 - 1), r1 = chain ? h : min(h, y1 + 1);  // rows needed
         const int S = tail_stride(w);
-        if (c > 0) {  // a pyramid level: 16-byte aligned rows
-            const int C = (w + 15) / 16;
-            for (int i = threadIdx.x; i < (r1 - r0) * C; i += blockDim.x) {
-                const int y = r0 + i / C, k = i % C;
-                const uint4 v = reinterpret_cast<const uint4 *>(Lc.img + (size_t)y * Lc.pitch)[k];
-                uint32_t *d = reinterpret_cast<uint32_t *>(cur + y * S) + 1 + 4 * k;
-                const int room = S / 4 - 1 - 4 * k;  // words left in the row
-                if (room > 0) d[0] = v.x;
-                if (room > 1) d[1] = v.y;
-                if (room > 2) d[2] = v.z;
-                if (room > 3) d[3] = v.w;
-            }
-        } else {  // the caller's image: any alignment
-            const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-            for (int y = r0 + (threadIdx.x >> 5); y < r1; y += nw) {
-                const uint8_t *sr = src + (size_t)y * sp;
-                for (int x = lane; x < w; x += 32) {
-                    const uint8_t v = sr[x];
-                    cur[y * S + 4 + x] = v;
-                    if (chain && src != Lc.img) Lc.img[(size_t)y * Lc.pitch + x] = v;
-                }
+        const int C = (w + 15) / 16;
+        for (int i = threadIdx.x; i < (r1 - r0) * C; i += blockDim.x) {
+            const int y = r0 + i / C, k = i % C, n = min(16, w - 16 * k);
+            const uint8_t *q = src + (size_t)y * sp + 16 * k;  // (the caller's image: any alignment)
+            const uint4 v = c > 0 ? *reinterpret_cast<const uint4 *>(q) : load16_any(q, n);
+            uint32_t *d = reinterpret_cast<uint32_t *>(cur + y * S) + 1 + 4 * k;
+            const int room = S / 4 - 1 - 4 * k;  // words left in the row
+            if (room > 0) d[0] = v.x;
+            if (room > 1) d[1] = v.y;
+            if (room > 2) d[2] = v.z;
+            if (room > 3) d[3] = v.w;
+            if (c == 0 && chain && src != Lc.img) {  // the level-0 copy
+                uint8_t *o = Lc.img + (size_t)y * Lc.pitch + 16 * k;
+                const uint32_t vq[4] = {v.x, v.y, v.z, v.w};
+                if (n == 16)
+                    *reinterpret_cast<uint4 *>(o) = v;
+                else
+                    for (int b = 0; b < n; ++b) o[b] = (uint8_t)(vq[b >> 2] >> (8 * (b & 3)));
             }
         }
         __syncwarp();
