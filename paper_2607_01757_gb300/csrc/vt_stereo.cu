@@ -328,7 +328,7 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
         const double iz = recip(rz);
         const double dx = ur - fma(KR[0], rx * iz, KR[2]), dy = vr - fma(KR[1], ry * iz, KR[3]);
         const double d2 = fma(dx, dx, dy * dy), m2 = g.prm.min_disp * g.prm.min_disp;
-        if (!(fabs(d2 - m2) > fma(kBand, d2 + m2, 1e-9))) return false;
+        if (!(isinf(m2) ? d2 < m2 : fabs(d2 - m2) > fma(kBand, d2 + m2, 1e-9))) return false;
         if (d2 < m2) {
             o.reason = VT_LOST_DISP;
             return true;
@@ -358,7 +358,7 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
     const double exl = fma(KL[0], X * il, KL[2] - ul), eyl = fma(KL[1], Y * il, KL[3] - vl);
     const double exr = fma(KR[0], XR * ir, KR[2] - ur), eyr = fma(KR[1], YR * ir, KR[3] - vr);
     const double e2 = fmax(fma(exl, exl, eyl * eyl), fma(exr, exr, eyr * eyr)), m2 = g.prm.max_reproj * g.prm.max_reproj;
-    if (!(fabs(e2 - m2) > fma(kBand, e2 + m2, 1e-9))) return false;
+    if (!(isinf(m2) ? e2 < m2 : fabs(e2 - m2) > fma(kBand, e2 + m2, 1e-9))) return false;
     if (e2 > m2) {
         o.reason = VT_LOST_REPROJ;
         return true;
