@@ -223,8 +223,8 @@ __device__ __forceinline__ void jacobi_rotate32(float (&M)[4][4], float (&V)[4][
     }
 }
 
-// 1 / v to FP64 accuracy, from the FP32 reciprocal by two Newton steps (v
-// within FP32's range; not a number otherwise).
+// 1 / v to FP64 accuracy, from the FP32 reciprocal by two Newton steps.  |v| in
+// 1e-30 .. 1e30, which the callers see to: beyond FP32's range the result is 0.
 __device__ __forceinline__ double recip(double v) {
     double r = (double)__frcp_rn((float)v);
     r = fma(r, fma(-v, r, 1.0), r);
@@ -323,7 +323,7 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
     const double rx = fma(R[0], xl, fma(R[1], yl, R[2]));
     const double ry = fma(R[3], xl, fma(R[4], yl, R[5]));
     const double rz = fma(R[6], xl, fma(R[7], yl, R[8]));
-    if (!(fabs(rz) > 1e-6)) return false;
+    if (!(fabs(rz) > 1e-6 && fabs(rz) < 1e30)) return false;
     if (rz > 0.0) {
         const double iz = recip(rz);
         const double dx = ur - fma(KR[0], rx * iz, KR[2]), dy = vr - fma(KR[1], ry * iz, KR[3]);
@@ -354,6 +354,7 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
         return false;
     if (!(ZR > 0.0 && Z > g.prm.z_min && Z < g.prm.z_max)) return true;
     if (!(fabs(Z) > band)) return false;
+    if (!(fabs(Z) < 1e30 && fabs(ZR) < 1e30)) return false;
     const double il = recip(Z), ir = recip(ZR);
     const double exl = fma(KL[0], X * il, KL[2] - ul), eyl = fma(KL[1], Y * il, KL[3] - vl);
     const double exr = fma(KR[0], XR * ir, KR[2] - ur), eyr = fma(KR[1], YR * ir, KR[3] - vr);

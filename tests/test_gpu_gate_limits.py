@@ -78,3 +78,18 @@ def test_infinite_thresholds_time():
     with_bound = _us(pl, pr, rig, S.GateParams(1.0, 0.3, np.inf, 3.0))
     without = _us(pl, pr, rig, S.GateParams(1.0, 0.3, np.inf, np.inf))
     assert without < 2.0 * with_bound, (without, with_bound)
+
+
+@pytest.mark.parametrize("scale", [1e-39, 1e-20, 1e6, 1e20, 1e39])
+def test_rotation_out_of_range(scale):
+    """R and t scaled together describe the same rig up to the scale of X_R: the
+    disparity is the unscaled one's (FP32 reciprocals and rotation angles must not
+    decide it)."""
+    pl, pr, rig = _pairs(2000, 0.11, 3, scale=scale)
+    pr[:50] = np.float32([rig.kr[2], rig.kr[3]])  # (the principal point: 0 / 0 where a ray's depth is lost)
+    prm = S.GateParams(20.0, 0.3, 50.0, 1.5)
+    r = S.stereo_gate(pl, pr, None, rig, prm)
+    _, _, rs = _gpu_gate(pl, pr, None, rig, prm)
+    far = np.abs(r.disparity - prm.min_disp) > MARGIN
+    assert (50 < (r.reason == S.GATE_DISP).sum() < 1950)
+    assert ((rs == S.GATE_DISP) == (r.reason == S.GATE_DISP))[far].all()
