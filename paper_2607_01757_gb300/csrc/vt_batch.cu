@@ -520,8 +520,7 @@ vt_status vt_batch_set_gates(vt_batch *b, const vt_gate_task *gates, int ngates,
     for (int i = 0; i < ngates; ++i) {
         const vt_gate_task &g = gates[i];
         gt[i].rig = g.rig;
-        gt[i].inv[0] = 1.0 / g.rig.kl[0], gt[i].inv[1] = 1.0 / g.rig.kl[1];
-        gt[i].inv[2] = 1.0 / g.rig.kr[0], gt[i].inv[3] = 1.0 / g.rig.kr[1];
+        gt[i].k = gate_scale(g.rig);
         gt[i].pts_l = reinterpret_cast<const float2 *>(g.pts_l);
         gt[i].pts_r = reinterpret_cast<const float2 *>(g.pts_r);
         gt[i].status_in = g.status_in;

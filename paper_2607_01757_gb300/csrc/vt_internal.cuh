@@ -202,10 +202,21 @@ struct BTask {
     int n, fb, p0, levels;
 };
 
+// Constants of a stereo rig for the gate (see gate_fast, vt_stereo.cu).
+struct GateScale {
+    double ikl[2], ikr[2];  // 1 / fx, 1 / fy of both cameras
+    double unit, beta;      // power of two of the translation's size (1 below 2), and 1 / unit^2
+    double t[3];            // the translation / unit
+    float rows;             // largest sum of absolute values of a row of R, at least 1
+    float px;               // largest focal length plus largest principal point coordinate
+    int fast;               // 0: the rig goes to the FP64 route alone
+};
+GateScale gate_scale(const vt_stereo_rig &rig);
+
 // One stereo-gate task of a batched run: a rig and the pairs it checks.
 struct GTask {
     vt_stereo_rig rig;
-    double inv[4];  // 1 / fx, 1 / fy of the left and the right camera
+    GateScale k;
     const float2 *pts_l, *pts_r;
     const uint8_t *status_in;
     float *xyz;

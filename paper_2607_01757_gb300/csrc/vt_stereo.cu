@@ -2,7 +2,8 @@
 // correspondences (Sec. III-C: negligible-disparity matches are dropped, the
 // rest triangulated with the rig's extrinsics and kept only with a positive
 // depth inside a valid range and at most 1.5 px of reprojection error in
-// both views).  One thread per correspondence, FP64 throughout:
+// both views).  One thread per correspondence; decisions and points are FP64's
+// (the eigenvectors are found in FP32 and refined, see gate_fast):
 //
 //   disparity  |p_R - pi_R(R K_L^-1 p_L)| (image of the left ray's point at
 //              infinity in the right view; infinite when it lies behind the
@@ -23,16 +24,38 @@ namespace vt {
 
 constexpr int kJacobiSweeps = 12;
 
+// Rigs with a shorter translation go to the FP64 route alone: the spectrum's gap
+// shrinks with its square (at 0.016 to 5e-5 of the largest eigenvalue, where half
+// of the pairs are left to that route anyway).
+constexpr double kGateMinT = 0.015625;
+
 struct GateArgs {
     vt_stereo_rig rig;
     vt_gate_params prm;
-    double ikl[2], ikr[2];  // 1 / fx, 1 / fy of both cameras
-
-    __host__ __device__ void inverses() {
-        ikl[0] = 1.0 / rig.kl[0], ikl[1] = 1.0 / rig.kl[1];
-        ikr[0] = 1.0 / rig.kr[0], ikr[1] = 1.0 / rig.kr[1];
-    }
+    GateScale k;
 };
+
+// The constants of a rig that the fast route uses.
+GateScale gate_scale(const vt_stereo_rig &rig) {
+    GateScale k;
+    k.ikl[0] = 1.0 / rig.kl[0], k.ikl[1] = 1.0 / rig.kl[1];
+    k.ikr[0] = 1.0 / rig.kr[0], k.ikr[1] = 1.0 / rig.kr[1];
+    const double t = std::fmax(std::fabs(rig.t[0]), std::fmax(std::fabs(rig.t[1]), std::fabs(rig.t[2])));
+    k.unit = t >= 2.0 ? std::ldexp(1.0, std::ilogb(t)) : 1.0;
+    k.beta = 1.0 / k.unit / k.unit;
+    for (int i = 0; i < 3; ++i) k.t[i] = rig.t[i] / k.unit;
+    double r = 1.0, f = 0.0, c = 0.0;
+    for (int i = 0; i < 3; ++i)
+        r = std::fmax(r, std::fabs(rig.R[3 * i]) + std::fabs(rig.R[3 * i + 1]) + std::fabs(rig.R[3 * i + 2]));
+    for (int i = 0; i < 2; ++i) {
+        f = std::fmax(f, std::fmax(std::fabs(rig.kl[i]), std::fabs(rig.kr[i])));
+        c = std::fmax(c, std::fmax(std::fabs(rig.kl[2 + i]), std::fabs(rig.kr[2 + i])));
+    }
+    k.rows = (float)r;
+    k.px = (float)(f + c);
+    k.fast = t >= kGateMinT;
+    return k;
+}
 
 // One Jacobi rotation in the (P, Q) plane of the symmetric M (upper
 // triangle M[i][j], i < j, and the diagonal are kept), accumulating V.
@@ -183,16 +206,28 @@ __device__ __forceinline__ GateOut gate_point(const GateArgs &g, float2 pl, floa
 //     sum_k -(v_k . r) / (l_k - l_0) v_k from the FP32 eigenpairs.  A step
 //     shrinks the error by the relative error of those (about 1e-6 |A|^2 /
 //     (l_1 - l_0)); the steps end when the next one, judged by the last two,
-//     is below 1e-13: usually after two;
+//     is below the rounding (`err` below): usually after two;
 //   - one reciprocal serves the divisions by the same number, and distances are
 //     compared squared.
-// A pair is left to gate_point when the refinement has not converged, when the
-// spectrum has no gap, or when any decision lies within 1e-8 (relative) of its
-// threshold -- a million times the rounding of either route -- so both take
-// the same decisions.  Not-a-numbers fail these tests and go there, too.
-// Measured: 19,000 pairs 78 -> 11.4 us, about 6,000 pairs of a batched run 76 ->
-// 14.7 us (one warp a CTA spreads them; cold caches); no pair of either is left
-// to gate_point.
+// The unit that minimises |A x| is the one in the rig's own unit of length, but it
+// is sought in coordinates whose last column is scaled by a power of two to the
+// translation's size (y_4 = unit x_4, |x|^2 = y_1^2 + y_2^2 + y_3^2 + y_4^2 /
+// unit^2): gap and stop then mean the same for a rig in millimetres.  Without it
+// the gap shrank with the square of the translation, and from 250 on every pair
+// went through both routes (19,000 pairs at 250: 68 us, 13.0 so; 12.1 at 0.11).
+//
+// The null vector's error is at most `err` = 2e-15 l_3 / (l_1 - l_0) + 1e-15 for
+// the rounding of the residual (an FP64 row of four terms is off by 4 2^-53
+// |A_i|, the squares of the |A_i| add up to at most 4 l_3, and the gap carries
+// that to the vector) and as much again for the refinement's stop; the point's is
+// `rel` (unit + |X|), rel = 4 err / |y_4|, a factor of two to spare.  A pair is
+// left to gate_point when the refinement has not converged, when the spectrum has
+// no gap, when rel passes 1e-7 (points beyond some 1e4 to 1e7 translations), or
+// when a decision lies within that error of its threshold (at least 1e-8,
+// relative, for depths).  Not-a-numbers fail these tests and go there, too.
+// Measured: 19,000 pairs 78 -> 11.8 us, about 6,000 pairs of a batched run 76 ->
+// 14.7 us (one warp a CTA spreads them; cold caches); hardly a pair of either is
+// left to gate_point.
 
 // One FP32 Jacobi rotation in the (P, Q) plane (see jacobi_rotate).
 template <int P, int Q>
@@ -223,18 +258,21 @@ __device__ __forceinline__ void jacobi_rotate32(float (&M)[4][4], float (&V)[4][
     }
 }
 
-// 1 / v to FP64 accuracy, from the FP32 reciprocal by two Newton steps.  |v| in
-// 1e-30 .. 1e30, which the callers see to: beyond FP32's range the result is 0.
-__device__ __forceinline__ double recip(double v) {
-    double r = (double)__frcp_rn((float)v);
+// 1 / v to FP64 accuracy, from the FP32 reciprocal `seed` by two Newton steps.
+// Beyond FP32's range both are 0: the callers test the seed (kSeedMin).
+constexpr float kSeedMin = 1e-30f;
+__device__ __forceinline__ double recip(double v, float &seed) {
+    seed = __frcp_rn((float)v);
+    double r = (double)seed;
     r = fma(r, fma(-v, r, 1.0), r);
     return fma(r, fma(-v, r, 1.0), r);
 }
 
 // The null vector of the rows (-1, 0, xl, 0), (0, -1, yl, 0), a and b: the unit
 // x that minimises |A x|, or false (see above).
+// x: in scaled coordinates (a[3], b[3] scaled; beta = 1 / unit^2); err: its error.
 __device__ __forceinline__ bool null_vector_fast(double xl, double yl, const double (&a)[4], const double (&b)[4],
-                                                 double (&x)[4]) {
+                                                 double beta, double (&x)[4], float &err) {
     constexpr int kSweeps = 4, kSteps = 8;
     float m[4][4], V[4][4];
     {
@@ -278,6 +316,7 @@ __device__ __forceinline__ bool null_vector_fast(double xl, double yl, const dou
         }
     const float top = fmaxf(fmaxf(l[1], l[2]), l[3]), gap = fminf(fminf(l[1], l[2]), l[3]) - l[0];
     if (!(gap > 2e-5f * top)) return false;
+    err = fmaf(2e-15f, top / gap, 1e-15f);
     const float w[3] = {1.0f / (l[0] - l[1]), 1.0f / (l[0] - l[2]), 1.0f / (l[0] - l[3])};
     const float n0 = rsqrtf(fmaf(V[0][0], V[0][0], fmaf(V[1][0], V[1][0], fmaf(V[2][0], V[2][0], V[3][0] * V[3][0]))));
 #pragma unroll
@@ -288,12 +327,18 @@ __device__ __forceinline__ bool null_vector_fast(double xl, double yl, const dou
         const double e0 = fma(xl, x[2], -x[0]), e1 = fma(yl, x[2], -x[1]);
         const double e2 = fma(a[0], x[0], fma(a[1], x[1], fma(a[2], x[2], a[3] * x[3])));
         const double e3 = fma(b[0], x[0], fma(b[1], x[1], fma(b[2], x[2], b[3] * x[3])));
-        // |x| is 1 within 1e-6, and what that leaves of rho x in r is along x
-        const double rho = fma(e0, e0, fma(e1, e1, fma(e2, e2, e3 * e3)));
+        // (unscaled, |x| is 1 within 1e-6, and what that leaves of rho x in r is along x)
+        double rho = fma(e0, e0, fma(e1, e1, fma(e2, e2, e3 * e3)));
+        double rb = rho;
+        if (beta != 1.0) {
+            float seed;
+            rho *= recip(fma(x[0], x[0], fma(x[1], x[1], fma(x[2], x[2], beta * (x[3] * x[3])))), seed);
+            rb = rho * beta;
+        }
         const float r[4] = {(float)fma(a[0], e2, fma(b[0], e3, fma(-rho, x[0], -e0))),
                             (float)fma(a[1], e2, fma(b[1], e3, fma(-rho, x[1], -e1))),
                             (float)fma(a[2], e2, fma(b[2], e3, fma(xl, e0, fma(yl, e1, -rho * x[2])))),
-                            (float)fma(a[3], e2, fma(b[3], e3, -rho * x[3]))};
+                            (float)fma(a[3], e2, fma(b[3], e3, -rb * x[3]))};
         float d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
@@ -304,42 +349,49 @@ __device__ __forceinline__ bool null_vector_fast(double xl, double yl, const dou
 #pragma unroll
         for (int i = 0; i < 4; ++i) x[i] += (double)d[i];
         const float step = fmaxf(fmaxf(fabsf(d[0]), fabsf(d[1])), fmaxf(fabsf(d[2]), fabsf(d[3])));
-        if (!(step < 0.1f * last)) return step < 1e-14f;  // does not shrink (or has reached the rounding)
-        if (k > 0 && step * step < 1e-13f * last) return true;
+        if (!(step < 0.1f * last)) return step < err;  // does not shrink (or has reached the rounding)
+        if (k > 0 && step * step < err * last) return true;
         last = step;
     }
     return false;
 }
 
+// Whether v >= 0 is infinite.
+__device__ __forceinline__ bool infinite(double v) { return __double2hiint(v) == 0x7ff00000; }
+
 // gate_point's result, or false when the pair is to be left to it.
 __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 pr, bool tracked, GateOut &o) {
     o = {0.f, 0.f, 0.f, 0, VT_LOST_INPUT};
     if (!tracked || !isfinite(pl.x) || !isfinite(pl.y) || !isfinite(pr.x) || !isfinite(pr.y)) return true;
-    constexpr double kBand = 1e-8;  // relative distance from a threshold below which gate_point decides
-    const double *KL = g.rig.kl, *KR = g.rig.kr, *R = g.rig.R, *T = g.rig.t;
+    const double *KL = g.rig.kl, *KR = g.rig.kr, *R = g.rig.R, *T = g.rig.t, *t = g.k.t;
     const double ul = pl.x, vl = pl.y, ur = pr.x, vr = pr.y;
-    const double xl = (ul - KL[2]) * g.ikl[0], yl = (vl - KL[3]) * g.ikl[1];
-    const double xr = (ur - KR[2]) * g.ikr[0], yr = (vr - KR[3]) * g.ikr[1];
+    const double xl = (ul - KL[2]) * g.k.ikl[0], yl = (vl - KL[3]) * g.k.ikl[1];
+    const double xr = (ur - KR[2]) * g.k.ikr[0], yr = (vr - KR[3]) * g.k.ikr[1];
     const double rx = fma(R[0], xl, fma(R[1], yl, R[2]));
     const double ry = fma(R[3], xl, fma(R[4], yl, R[5]));
     const double rz = fma(R[6], xl, fma(R[7], yl, R[8]));
-    if (!(fabs(rz) > 1e-6 && fabs(rz) < 1e30)) return false;
+    float seed;
+    if (!(fabs(rz) > 1e-6)) return false;
     if (rz > 0.0) {
-        const double iz = recip(rz);
+        const double iz = recip(rz, seed);
+        if (!(seed > kSeedMin)) return false;
         const double dx = ur - fma(KR[0], rx * iz, KR[2]), dy = vr - fma(KR[1], ry * iz, KR[3]);
         const double d2 = fma(dx, dx, dy * dy), m2 = g.prm.min_disp * g.prm.min_disp;
-        if (!(isinf(m2) ? d2 < m2 : fabs(d2 - m2) > fma(kBand, d2 + m2, 1e-9))) return false;
+        if (!(infinite(m2) ? d2 < m2 : fabs(d2 - m2) > fma(1e-8, d2 + m2, 1e-9))) return false;
         if (d2 < m2) {
             o.reason = VT_LOST_DISP;
             return true;
         }
     }
-    const double a[4] = {fma(xr, R[6], -R[0]), fma(xr, R[7], -R[1]), fma(xr, R[8], -R[2]), fma(xr, T[2], -T[0])};
-    const double b[4] = {fma(yr, R[6], -R[3]), fma(yr, R[7], -R[4]), fma(yr, R[8], -R[5]), fma(yr, T[2], -T[1])};
+    const double a[4] = {fma(xr, R[6], -R[0]), fma(xr, R[7], -R[1]), fma(xr, R[8], -R[2]), fma(xr, t[2], -t[0])};
+    const double b[4] = {fma(yr, R[6], -R[3]), fma(yr, R[7], -R[4]), fma(yr, R[8], -R[5]), fma(yr, t[2], -t[1])};
     double x[4];
-    if (!null_vector_fast(xl, yl, a, b, x)) return false;
-    if (!(fabs(x[3]) > 1e-6)) return false;  // near infinity
-    const double iw = recip(x[3]);
+    float err;
+    if (!null_vector_fast(xl, yl, a, b, g.k.beta, x, err)) return false;
+    double iw = recip(x[3], seed);
+    const float rel = 4.0f * err * fabsf(seed);
+    if (!(rel < 1e-7f)) return false;  // near infinity
+    if (g.k.beta != 1.0) iw *= g.k.unit;
     const double X = x[0] * iw, Y = x[1] * iw, Z = x[2] * iw;
     o.x = (float)X;
     o.y = (float)Y;
@@ -348,18 +400,28 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
     const double XR = fma(R[0], X, fma(R[1], Y, fma(R[2], Z, T[0])));
     const double YR = fma(R[3], X, fma(R[4], Y, fma(R[5], Z, T[1])));
     const double ZR = fma(R[6], X, fma(R[7], Y, fma(R[8], Z, T[2])));
-    const double band = kBand * (fabs(X) + fabs(Y) + fabs(Z) + 1.0);
+    const double size = fabs(X) + fabs(Y) + fabs(Z) + g.k.unit;
+    const double band = (double)(fmaxf(1e-8f, rel) * g.k.rows) * size;
     if (!(fabs(ZR) > band) || !(Z < g.prm.z_min - band || Z > g.prm.z_min + band) ||
         !(Z < g.prm.z_max - band || Z > g.prm.z_max + band))
         return false;
     if (!(ZR > 0.0 && Z > g.prm.z_min && Z < g.prm.z_max)) return true;
     if (!(fabs(Z) > band)) return false;
-    if (!(fabs(Z) < 1e30 && fabs(ZR) < 1e30)) return false;
-    const double il = recip(Z), ir = recip(ZR);
+    float sl, sr;
+    const double il = recip(Z, sl), ir = recip(ZR, sr);
+    sl = fabsf(sl);
+    if (!(fminf(sl, sr) > kSeedMin)) return false;
     const double exl = fma(KL[0], X * il, KL[2] - ul), eyl = fma(KL[1], Y * il, KL[3] - vl);
     const double exr = fma(KR[0], XR * ir, KR[2] - ur), eyr = fma(KR[1], YR * ir, KR[3] - vr);
+    // An error e is off by at most d = rel size |R| / |Z| times f + f |X / Z|, and
+    // f |X / Z| by at most the observation's distance from the principal point
+    // and e.  e and the threshold m compare as their squares where those differ by
+    // more than d (e + m), which is at most d's factor (px + um + 2) (1 + e^2 + m^2).
+    const float um = fmaxf(fmaxf(fabsf(pl.x), fabsf(pl.y)), fmaxf(fabsf(pr.x), fabsf(pr.y)));
+    const float de = 2.0f * rel * (float)size * g.k.rows * fmaxf(sl, sr) * (g.k.px + um + 2.0f);
+    const double tol = (double)fmaxf(de, 1e-10f);
     const double e2 = fmax(fma(exl, exl, eyl * eyl), fma(exr, exr, eyr * eyr)), m2 = g.prm.max_reproj * g.prm.max_reproj;
-    if (!(isinf(m2) ? e2 < m2 : fabs(e2 - m2) > fma(kBand, e2 + m2, 1e-9))) return false;
+    if (!(infinite(m2) ? e2 < m2 : fabs(e2 - m2) > fma(tol, e2 + m2, tol))) return false;
     if (e2 > m2) {
         o.reason = VT_LOST_REPROJ;
         return true;
@@ -371,7 +433,7 @@ __device__ __forceinline__ bool gate_fast(const GateArgs &g, float2 pl, float2 p
 
 __device__ __forceinline__ GateOut gate(const GateArgs &g, float2 pl, float2 pr, bool tracked) {
     GateOut o;
-    if (!gate_fast(g, pl, pr, tracked, o)) o = gate_point(g, pl, pr, tracked);
+    if (!g.k.fast || !gate_fast(g, pl, pr, tracked, o)) o = gate_point(g, pl, pr, tracked);
     return o;
 }
 
@@ -415,7 +477,7 @@ __global__ void __launch_bounds__(GATE_THREADS) k_gate_batch(const uint8_t *tab)
         GateArgs g;
         g.rig = t.rig;
         g.prm = H->G;
-        g.ikl[0] = t.inv[0], g.ikl[1] = t.inv[1], g.ikr[0] = t.inv[2], g.ikr[1] = t.inv[3];
+        g.k = t.k;
         const GateOut o = gate(g, t.pts_l[i], t.pts_r[i], t.status_in ? t.status_in[i] != 0 : true);
         if (t.xyz) {
             t.xyz[3 * i + 0] = o.x;
@@ -458,7 +520,7 @@ extern "C" vt_status vt_stereo_gate(const float *pts_l, const float *pts_r, cons
     GateArgs g;
     g.rig = *rig;
     g.prm = *prm;
-    g.inverses();
+    g.k = gate_scale(*rig);
     const cudaError_t e = launch_pdl(k_stereo_gate, (n + GATE_THREADS - 1) / GATE_THREADS, GATE_THREADS, 0,
                                      (cudaStream_t)cuda_stream, true, reinterpret_cast<const float2 *>(pts_l),
                                      reinterpret_cast<const float2 *>(pts_r), status_in, n, g, xyz_out, status_out,

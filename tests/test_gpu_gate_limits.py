@@ -93,3 +93,56 @@ def test_rotation_out_of_range(scale):
     far = np.abs(r.disparity - prm.min_disp) > MARGIN
     assert (50 < (r.reason == S.GATE_DISP).sum() < 1950)
     assert ((rs == S.GATE_DISP) == (r.reason == S.GATE_DISP))[far].all()
+
+
+def _points(pl, pr, rig):
+    """The triangulated points to better than 1e-9 of their distance whatever the
+    rig's unit: inverse iteration on the generalised problem, the last coordinate
+    scaled to the translation, from the FP64 SVD's vector."""
+    L, Q = pl.astype(np.float64), pr.astype(np.float64)
+    xl = (L - rig.kl[2:]) / rig.kl[:2]
+    xr = (Q - rig.kr[2:]) / rig.kr[:2]
+    x = S.triangulate_dlt(xl, xr, rig.R, rig.t)
+    unit = np.linalg.norm(rig.t)
+    o, z = np.ones(len(pl)), np.zeros(len(pl))
+    P = np.concatenate([rig.R, rig.t[:, None] / unit], 1)
+    A = np.stack([np.stack([-o, z, xl[:, 0], z], 1), np.stack([z, -o, xl[:, 1], z], 1), xr[:, :1] * P[2] - P[0],
+                  xr[:, 1:] * P[2] - P[1]], 1)
+    B = np.array([1.0, 1.0, 1.0, unit**-2])
+    y = x * np.array([1.0, 1.0, 1.0, unit])
+    M = np.einsum("nri,nrj->nij", A, A)
+    for _ in range(3):
+        lam = ((A @ y[..., None])[..., 0]**2).sum(1) / (B * y * y).sum(1)
+        K = M - 0.999 * lam[:, None, None] * np.diag(B)
+        y = np.linalg.solve(K, (B * y)[..., None])[..., 0]
+        y /= np.linalg.norm(y, axis=1)[:, None]
+    return unit * y[:, :3] / y[:, 3:]
+
+
+BASELINES = [1e-3, 0.015, 0.016, 0.11, 1.9, 2.0, 11.0, 110.0, 250.0, 1000.0, 3e4]
+
+
+@pytest.mark.parametrize("baseline", BASELINES)
+@pytest.mark.parametrize("depth", [600.0, 5e4])
+def test_units(baseline, depth):
+    """The same scene in any unit of length, near and far.  The fast route's points
+    are off by at most its guard, 3e-8 of their distance, besides the output's
+    rounding; a pair in a thousand may be left to the other route (whose error
+    grows with the translation)."""
+    n = 5000
+    pl, pr, rig = _pairs(n, baseline, int(depth), depth=depth, noise=0.4 if depth < 1e3 else 0.002)
+    r, xyz, rs = _same(pl, pr, rig, S.GateParams(0.0, 0.0, np.inf, 1.5))
+    if baseline < 0.0157:  # the FP64 route alone
+        return
+    X = _points(pl, pr, rig)
+    tri = (rs == S.GATE_OK) | (rs == S.GATE_DEPTH) | (rs == S.GATE_REPROJ)
+    tri &= (np.abs(X) < 1e5 * baseline).all(1)  # (noise puts far points anywhere; beyond the guard there is the other route)
+    tol = 2.0**-24 * np.abs(X) + 3e-8 * (2.0 * baseline + np.abs(X).sum(1))[:, None]
+    off = (np.abs(xyz - X) > tol).any(1) & tri
+    assert tri.sum() > 0.5 * n and off.sum() <= 0.001 * n, (off.sum(), (np.abs(xyz - X) / tol)[tri].max())
+
+
+def test_units_time():
+    """... and in the same time."""
+    us = {b: _us(*_pairs(200000, b, 5), S.GateParams(1.0, 0.1 * b, 500.0 * b, 1.5)) for b in (0.11, 110.0, 500.0, 3e4)}
+    assert all(v < 1.5 * us[0.11] for v in us.values()), us
