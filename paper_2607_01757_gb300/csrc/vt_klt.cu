@@ -67,7 +67,7 @@ __global__ void k_fb_check(const float2 *p0, const float2 *p1, const uint8_t *sf
     if (i >= n) return;
     const float2 a = p0[i], b = p1[i];
     const float dx = a.x - b.x, dy = a.y - b.y;
-    out[i] = (uint8_t)(sf[i] && sb[i] && (dx * dx + dy * dy <= thr2));
+    out[i] = (uint8_t)(sf[i] && sb[i] && (norm2(dx, dy) <= thr2));
 }
 
 template <int WIN, int GT, bool FB, bool F64>

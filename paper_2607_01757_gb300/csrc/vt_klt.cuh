@@ -167,6 +167,11 @@ __device__ __forceinline__ float kdiff(float a, float b, float c, float d) {
     return fmaf(a, b, -w) - fmaf(c, d, -w);
 }
 
+// x^2 + y^2, rounded the same wherever it decides something: left to the
+// compiler, which of the products is fused is each kernel's own, and a point's
+// result would depend on the kernel that tracked it.
+__device__ __forceinline__ float norm2(float x, float y) { return fmaf(x, x, __fmul_rn(y, y)); }
+
 // 2^-l exactly.
 __device__ __forceinline__ float pow2neg(int l) { return __int_as_float((127 - l) << 23); }
 
@@ -997,7 +1002,7 @@ __device__ __forceinline__ void track_point(const Level *I, const Level *J, cons
             nux += ex;
             nuy += ey;
             ++o.iters;
-            if (ex * ex + ey * ey < P.eps2 || k >= P.max_iters) break;
+            if (norm2(ex, ey) < P.eps2 || k >= P.max_iters) break;
             const float qx = qx0 + nux, qy = qy0 + nuy;
             bx = qx - cfx, by = qy - cfy;
             if (max(__float_as_uint(bx), __float_as_uint(by)) >= cell_end) {
@@ -1116,7 +1121,7 @@ __device__ __forceinline__ void track_point_dir(const Level *I, const Level *J, 
                 return;
             }
             const float dx = ux0 - r.x, dy = uy0 - r.y;
-            if (!(dx * dx + dy * dy <= P.fb_thr2)) {
+            if (!(norm2(dx, dy) <= P.fb_thr2)) {
                 o.status = 0;
                 o.reason = VT_LOST_FB;
             }
