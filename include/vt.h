@@ -291,7 +291,7 @@ typedef struct vt_gftt vt_gftt; /* opaque: workspace for levels up to max_w x ma
 VT_API vt_status vt_gftt_create(int max_w, int max_h, vt_gftt **out);
 
 /* Workspace for vt_gftt_detect_many: the levels of one call may hold up to
- * max_pixels pixels together (about 50 bytes of device memory per pixel). */
+ * max_pixels pixels together (16.1 bytes of device memory per pixel). */
 VT_API vt_status vt_gftt_create_pixels(long long max_pixels, vt_gftt **out);
 
 /* Detect corners on level `level` of `p`.  mask_pts: device float2[n_mask]
